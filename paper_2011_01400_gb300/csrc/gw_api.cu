@@ -185,7 +185,8 @@ struct SurState {
   double* d_Sc_d = nullptr;    // [sig_rows][nc]
   // q-group buffers of the surrogate pass
   int qbs = 0;
-  c128 *g_chi0 = nullptr, *g_E = nullptr, *g_work = nullptr, *g_A = nullptr, *g_U = nullptr;
+  uint8_t* g_work = nullptr;
+  c128 *g_chi0 = nullptr, *g_E = nullptr, *g_A = nullptr, *g_U = nullptr;
   float *d_d = nullptr, *d_x = nullptr, *d_sig = nullptr, *d_g = nullptr, *d_coef = nullptr;
 };
 
@@ -274,7 +275,7 @@ struct gw_plan_s {
   c128* d_chi0 = nullptr;   // [nw][N][N]
   c128* d_E = nullptr;      // [nw][N][N] eps~ then eps~^-1 - 1
   c128* d_Wc = nullptr;     // [nw][N][N]
-  c128* d_work = nullptr;   // [nw][N][N]
+  c128* d_work = nullptr;   // [nw][N][N], or the workspace of nw inversions where that is larger
   c128* d_tmp = nullptr;    // [nw][N][N]
   c128* d_sigma = nullptr;  // [NK][nsig][nw]
   double* d_head = nullptr; // [nw]
@@ -333,7 +334,8 @@ struct gw_plan_s {
   c64* d_Vh32 = nullptr;      // FP32 copies of V^1/2 for the split-precision screen
   c64* d_Vb32 = nullptr;
   // q-group buffers of gw_g0w0
-  c128 *g_chi0 = nullptr, *g_E = nullptr, *g_work = nullptr;
+  c128 *g_chi0 = nullptr, *g_E = nullptr;
+  uint8_t* g_work = nullptr;
   int qb = 0;
   double group_budget = 8.0e9;  // bytes for the q-group buffers of gw_g0w0
   MgenTuner mtune;              // picks the thread mapping of the fp32 M kernels per call shape
@@ -798,7 +800,7 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
   ALLOC(P->d_chi0, NN * nw);
   ALLOC(P->d_E, NN * nw);
   ALLOC(P->d_Wc, NN * nw);
-  ALLOC(P->d_work, NN * nw);
+  ALLOC(P->d_work, std::max(NN * nw, (inv_work_bytes(N, nw) + sizeof(c128) - 1) / sizeof(c128)));
   ALLOC(P->d_tmp, NN * nw);
   ALLOC(P->d_sigma, (size_t)P->NK * P->nsig * nw);
   ALLOC(P->d_head, nw);
@@ -1314,6 +1316,17 @@ gw_status herm_gemm(gw_plan_s* P, const c64* A, bool a_batch, const c128* H, boo
   return herm_gemm(P, A, a_batch, H, nullptr, h_batch, alpha, C, P->nw);
 }
 
+// E[b] := E[b]^{-1} - 1 for `batch` matrices eps~ (FP64)
+gw_status invert(gw_plan_s* P, c128* E, int batch, void* work) {
+  std::string err;
+  const gw_status s = launch_inv_minus_I(P->N, E, batch, (long long)P->N * P->N, work, P->d_status, P->st, err);
+  if (s != GW_OK) {
+    P->err = 1;
+    return fail(s, "inversion of eps~: " + err);
+  }
+  return GW_OK;
+}
+
 // eps~(q) = 1 - V^1/2 chi0 V^1/2 (head and wings at q = 0) into E ([nw][N][N], FP64)
 gw_status eps_core(gw_plan_s* P, int q, const c128* chi0, c128* E) {
   cudaStream_t st = P->st;
@@ -1461,11 +1474,11 @@ gw_status g0w0_sur(gw_plan_s* P, c128* sig);  // the surrogate pass, defined bel
 gw_status ensure_groups(gw_plan_s* P) {
   if (P->g_chi0) return GW_OK;
   const long long slot = (long long)P->N * P->N * P->nw;
-  const double per_q = 3.0 * sizeof(c128) * (double)slot;
+  const double per_q = 2.0 * sizeof(c128) * (double)slot + (double)inv_work_bytes(P->N, P->nw);
   P->qb = (int)std::max(1.0, std::min((double)P->NK, std::floor(P->group_budget / per_q)));
   GW_TRY(dalloc(P, &P->g_chi0, (size_t)slot * P->qb));
   GW_TRY(dalloc(P, &P->g_E, (size_t)slot * P->qb));
-  GW_TRY(dalloc(P, &P->g_work, (size_t)slot * P->qb));
+  GW_TRY(dalloc(P, &P->g_work, inv_work_bytes(P->N, P->nw * P->qb)));
   return GW_OK;
 }
 
@@ -1513,7 +1526,7 @@ gw_status g0w0_qlist(gw_plan_s* P, const std::vector<int>& qs_in, c128* sig_out,
     GW_TRY(chi0_prepare(P, q, nq));
     for (int j = 0; j < nq; ++j) GW_TRY(chi0_core(P, q[j], P->g_chi0 + j * slot));
     for (int j = 0; j < nq; ++j) GW_TRY(eps_core(P, q[j], P->g_chi0 + j * slot, P->g_E + j * slot));
-    launch_chol_inv_minus_I(N, P->g_E, nq * nw, NN, P->g_work, P->d_status, st);
+    GW_TRY(invert(P, P->g_E, nq * nw, P->g_work));
     for (int j = 0; j < nq; ++j)
       if (q[j] == 0 && P->p.head_wings == 2) GW_TRY(q0_average(P, P->g_E + j * slot));
     for (int j = 0; j < nq; ++j) GW_TRY(w_core(P, q[j], P->g_E + j * slot, P->g_chi0 + j * slot));
@@ -1566,7 +1579,7 @@ gw_status gw_screen(gw_plan P, int32_t sys, int32_t q, gw_complex* wc_out) {
   const long long NN = (long long)P->N * P->N;
   GW_TRY(eps_core(P, q, P->d_chi0, P->d_E));
   GW_CUDA(cudaMemsetAsync(P->d_status, 0, sizeof(int), st));
-  launch_chol_inv_minus_I(P->N, P->d_E, P->nw, NN, P->d_work, P->d_status, st);
+  GW_TRY(invert(P, P->d_E, P->nw, P->d_work));
   if (q == 0 && P->p.head_wings == 2) GW_TRY(q0_average(P, P->d_E));
   GW_TRY(w_core(P, q, P->d_E, P->d_Wc));
   GW_TRY(read_status(P, "gw_screen"));
@@ -1963,11 +1976,12 @@ gw_status g0w0_sur(gw_plan_s* P, c128* sig) {
   const long long NN = (long long)N * N;
   const long long slot = NN * nc;
   if (!S.g_chi0) {
-    const double per_q = 3.0 * sizeof(c128) * (double)slot + sizeof(c128) * (double)(NN + (long long)N * k);
+    const double per_q = 2.0 * sizeof(c128) * (double)slot + (double)inv_work_bytes(N, nc) +
+                         sizeof(c128) * (double)(NN + (long long)N * k);
     S.qbs = (int)std::max(1.0, std::min({(double)P->NK, std::floor(6.0e9 / per_q), std::floor(4096.0 / k)}));
     GW_TRY(dalloc(P, &S.g_chi0, (size_t)slot * S.qbs));
     GW_TRY(dalloc(P, &S.g_E, (size_t)slot * S.qbs));
-    GW_TRY(dalloc(P, &S.g_work, (size_t)slot * S.qbs));
+    GW_TRY(dalloc(P, &S.g_work, inv_work_bytes(N, nc * S.qbs)));
     GW_TRY(dalloc(P, &S.g_A, (size_t)NN * S.qbs));
     GW_TRY(dalloc(P, &S.g_U, (size_t)N * k * S.qbs));
     const size_t rows = (size_t)S.qbs * k;
@@ -1992,7 +2006,7 @@ gw_status g0w0_sur(gw_plan_s* P, c128* sig) {
         GW_CUDA(cudaMemcpyAsync(S.g_A + j * NN, S.g_E + j * slot, sizeof(c128) * NN, cudaMemcpyDeviceToDevice, st));
       }
       launch_axpby_identity<double>(N, S.g_A, NN, nq, -1.0, st);
-      launch_chol_inv_minus_I(N, S.g_E, nq * nc, NN, S.g_work, P->d_status, st);
+      GW_TRY(invert(P, S.g_E, nq * nc, S.g_work));
       GW_TRY(modes_core(P, S.g_A, NN, nq, S.g_U, (long long)N * k));
       mode_diag(P, S.g_E, slot, nc, nq, S.g_U, (long long)N * k, S.d_d, nc);
       launch_sur_inputs(nq * k, nc, S.d_d, S.d_x, S.d_sig, st);
@@ -2107,7 +2121,7 @@ gw_status gw_surrogate_modes(gw_plan P, int32_t sys, int32_t q, float* d_out, do
   GW_TRY(eps_core(P, q, P->d_chi0, P->d_E));
   GW_CUDA(cudaMemcpyAsync(S.d_A1, P->d_E + S.coarse[0] * NN, sizeof(c128) * NN, cudaMemcpyDeviceToDevice, st));
   launch_axpby_identity<double>(N, S.d_A1, NN, 1, -1.0, st);
-  launch_chol_inv_minus_I(N, P->d_E, nw, NN, P->d_work, P->d_status, st);
+  GW_TRY(invert(P, P->d_E, nw, P->d_work));
   GW_TRY(modes_core(P, S.d_A1, 0, 1, S.d_U1, 0));
   float* d = d_out ? d_out : reinterpret_cast<float*>(P->d_tmp);
   mode_diag(P, P->d_E, 0, nw, 1, S.d_U1, 0, d, nw);
@@ -2154,7 +2168,7 @@ gw_status gw_surrogate_data(gw_plan P, int32_t sys, float* x_out, float* y_out, 
                               cudaMemcpyDeviceToDevice, st));
     }
     launch_axpby_identity<double>(N, S.g_Af, NN, nq, -1.0, st);
-    launch_chol_inv_minus_I(N, P->g_E, nq * nw, NN, P->g_work, P->d_status, st);
+    GW_TRY(invert(P, P->g_E, nq * nw, P->g_work));
     GW_TRY(modes_core(P, S.g_Af, NN, nq, S.g_Uf, (long long)N * k));
     mode_diag(P, P->g_E, slot, nw, nq, S.g_Uf, (long long)N * k, S.d_df, nw);
     if (moments)

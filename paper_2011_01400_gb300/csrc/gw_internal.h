@@ -100,9 +100,11 @@ void launch_zgemm(int m, int n, int k, cplx<T> alpha, const cplx<T>* A, long lon
 template <typename T>
 void launch_chi0_simt(int N, int K, const cplx<T>* Mt, long long ldm, const float* delta_f, const double* delta_d,
                       const double* freq, int nw, double scale, c128* chi0, cudaStream_t st);
-// per matrix b: A[b] (Hermitian PD, row-major N x N, FP64) -> A[b] := A[b]^{-1} - I. Sets ST_NOT_PD.
-void launch_chol_inv_minus_I(int N, c128* A, int batch, long long stride, c128* work, int* status,
-                             cudaStream_t st);
+// k_inv.cu: per matrix b: A[b] (Hermitian PD, row-major N x N, FP64; its upper triangle is read)
+// -> A[b] := A[b]^{-1} - I. Sets ST_NOT_PD. work: inv_work_bytes(N, batch) bytes, 16-byte aligned.
+size_t inv_work_bytes(int N, int batch);
+gw_status launch_inv_minus_I(int N, c128* A, int batch, long long stride, void* work, int* status, cudaStream_t st,
+                             std::string& err);
 template <typename T> void launch_axpby_identity(int N, cplx<T>* A, long long s, int batch, T diag, cudaStream_t st);
 void launch_take_both(int N, const c128* C, long long s, int batch, float d, c64* X, c64* XH, cudaStream_t st);
 void launch_dev_identity(int N, const c64* T, long long total, unsigned* dev, cudaStream_t st);

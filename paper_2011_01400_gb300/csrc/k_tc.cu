@@ -480,6 +480,10 @@ gw_status launch_tc(const Maps& maps, const TcParams& p, cudaStream_t st, std::s
 
 }  // namespace
 
+bool tc_map_16bit(CUtensorMap* m, const void* base, long long ldk, long long rows, int box_rows, std::string& err) {
+  return make_map(m, base, 0, ldk, rows, box_rows, err);
+}
+
 bool tc_available() { return get_encode() != nullptr; }
 
 gw_status tc_sigma_run(const TcSigmaArgs& a, cudaStream_t st, std::string& err) {

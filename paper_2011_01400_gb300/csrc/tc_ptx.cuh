@@ -141,4 +141,9 @@ __device__ __forceinline__ float tf32_rn(float x) {
 __device__ __forceinline__ uint32_t bf2_bits(__nv_bfloat162 h) { return *reinterpret_cast<uint32_t*>(&h); }
 
 }  // namespace ptx
+
+// 2-D map over a row-major plane [rows][ldk] of 16-bit elements, box = 128 B of one row x box_rows
+// rows, 128-byte swizzle (k_tc.cu)
+bool tc_map_16bit(CUtensorMap* m, const void* base, long long ldk, long long rows, int box_rows, std::string& err);
+
 }  // namespace gw
