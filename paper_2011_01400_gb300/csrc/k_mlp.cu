@@ -65,111 +65,162 @@ Offs offsets(int I, int H, int O) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// C[M][N] = alpha * sum_k A(m,k) B(k,n) + beta * C + bias_scale * bias[n]
-//   A(m,k) = tA ? A[k*lda + m] : A[m*lda + k]   (fp32)
-//   B(k,n) = tB ? B[n*ldb + k] : B[k*ldb + n]   (fp32 or bf16, converted to fp32)
-// 64x64 tiles, k-steps of 16, 256 threads with 4x4 outputs each (strided by 16).
+// Dense products of the network, fp32 on CUDA cores: sum_k A(m,k) B(k,n) in ascending k,
+//   A(m,k) = TA ? A[k*lda + m] : A[m*lda + k]   (fp32)
+//   B(k,n) = BT ? B[n*ldb + k] : B[k*ldb + n]   (fp32 or bf16, converted to fp32)
+// with the layer's elementwise part in the epilogue:
+//   MM_PLAIN  C = alpha acc + bias[n]
+//   MM_SILU   C = acc + bias[n], X = silu(C)                        (forward layer)
+//   MM_DSILU  C = alpha acc silu'(X)                                (backward through a layer)
+//   MM_PART   C[z][m][0..N) = acc, C[z][m][N] = sum_k A(m,k) over k part z  (weight and bias gradients)
+// BM x 64 tiles (BM 128 or 64), 256 threads with BM/16 x 4 outputs each, k steps of 16 staged through
+// registers into two shared buffers. The FP32 units bound it: 8 x 4 outputs per thread need 3 128-bit
+// shared loads per 32 FMAs. The gradients reduce over the rows of the data set, M x N is one layer's
+// weights: the k range is split so that the chip is filled, and the parts are added in order.
+// 16384 rows, 12-256-256-256-48: loss and gradient 10.6 ms with 64 x 64 tiles of 4 x 4, one block per
+// output tile of a gradient and one thread per bias column; 0.74 ms now.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float sigm(float z) { return 1.f / (1.f + expf(-z)); }
 
-template <typename TB>
-__global__ void __launch_bounds__(256) k_mm(int M, int N, int K, const float* __restrict__ A, int lda, int tA,
-                                            const TB* __restrict__ B, int ldb, int tB, float* __restrict__ C, int ldc,
-                                            float alpha, float beta, const float* __restrict__ bias,
-                                            float bias_scale) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+enum { MM_PLAIN, MM_SILU, MM_DSILU, MM_PART };
+
+template <int BM, typename TB, bool TA, bool BT, int EPI>
+__global__ void __launch_bounds__(256) k_mm(int M, int N, int K, int kpart, const float* __restrict__ A, int lda,
+                                            const TB* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
+                                            float alpha, const float* __restrict__ bias, float* __restrict__ X) {
+  constexpr int AR = BM / 16, TMR = BM / 16;   // A elements staged per thread, outputs along m per thread
+  __shared__ __align__(16) float As[2][16][BM + 4];
+  __shared__ __align__(16) float Bs[2][16][64 + 4];
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * 64;
+  const int k0 = blockIdx.z * kpart, k1 = min(K, k0 + kpart);
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
+  float ra[AR], rb[4];
+  auto fetch = [&](int kb) {
+#pragma unroll
+    for (int r = 0; r < AR; ++r) {
+      const int e = tid + 256 * r;
+      const int mm = TA ? e % BM : e / 16, kk = TA ? e / BM : e % 16;
+      const int gm = m0 + mm, gk = kb + kk;
+      ra[r] = (gm < M && gk < k1) ? (TA ? A[(long long)gk * lda + gm] : A[(long long)gm * lda + gk]) : 0.f;
+    }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int e = tid + 256 * r;
-      int mm, kk;
-      if (tA) { kk = e / 64; mm = e % 64; } else { mm = e / 16; kk = e % 16; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      float va = 0.f;
-      if (gm < M && gk < K) va = tA ? A[(long long)gk * lda + gm] : A[(long long)gm * lda + gk];
-      As[kk][mm] = va;
-      int nn, kb;
-      if (tB) { nn = e / 16; kb = e % 16; } else { kb = e / 64; nn = e % 64; }
-      const int gn = n0 + nn, gk2 = k0 + kb;
-      float vb = 0.f;
-      if (gn < N && gk2 < K) vb = tB ? to_f(B[(long long)gn * ldb + gk2]) : to_f(B[(long long)gk2 * ldb + gn]);
-      Bs[kb][nn] = vb;
+      const int nn = BT ? e / 16 : e % 64, kk = BT ? e % 16 : e / 64;
+      const int gn = n0 + nn, gk = kb + kk;
+      rb[r] = (gn < N && gk < k1) ? to_f(BT ? B[(long long)gn * ldb + gk] : B[(long long)gk * ldb + gn]) : 0.f;
     }
-    __syncthreads();
+  };
+  auto stash = [&](int s) {
+#pragma unroll
+    for (int r = 0; r < AR; ++r) {
+      const int e = tid + 256 * r;
+      As[s][TA ? e / BM : e % 16][TA ? e % BM : e / 16] = ra[r];
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int e = tid + 256 * r;
+      Bs[s][BT ? e % 16 : e / 64][BT ? e / 16 : e % 64] = rb[r];
+    }
+  };
+  float acc[TMR][4] = {};
+  float csum = 0.f;                            // MM_PART: sum over k of A(m0 + tid, k), tid < BM
+  fetch(k0);
+  stash(0);
+  __syncthreads();
+  int s = 0;
+  for (int kb = k0; kb < k1; kb += 16) {
+    const bool more = kb + 16 < k1;
+    if (more) fetch(kb + 16);
 #pragma unroll
     for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
+      float a[TMR], b[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+      for (int i = 0; i < TMR; i += 4)
+        *reinterpret_cast<float4*>(a + i) = *reinterpret_cast<const float4*>(&As[s][kk][4 * ty + 16 * i]);
+      *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(&Bs[s][kk][4 * tx]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TMR; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
-    __syncthreads();
+    if constexpr (EPI == MM_PART) {
+      if (blockIdx.x == 0 && tid < BM)
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk) csum += As[s][kk][tid];
+    }
+    if (more) {
+      stash(s ^ 1);
+      __syncthreads();
+      s ^= 1;
+    }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 16 * i;
+  for (int i = 0; i < TMR; ++i) {
+    const int m = m0 + 4 * ty + 16 * (i & ~3) + (i & 3);
     if (m >= M) continue;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
+      const int n = n0 + 4 * tx + j;
       if (n >= N) continue;
-      float v = alpha * acc[i][j];
-      if (beta != 0.f) v += beta * C[(long long)m * ldc + n];
-      if (bias) v += bias_scale * bias[n];
-      C[(long long)m * ldc + n] = v;
+      if constexpr (EPI == MM_PART) {
+        C[((long long)blockIdx.z * M + m) * (N + 1) + n] = acc[i][j];
+      } else if constexpr (EPI == MM_DSILU) {
+        const float z = X[(long long)m * ldc + n], sg = sigm(z);
+        C[(long long)m * ldc + n] = alpha * acc[i][j] * sg * (1.f + z * (1.f - sg));
+      } else {
+        float v = alpha * acc[i][j];
+        if (bias) v += bias[n];
+        C[(long long)m * ldc + n] = v;
+        if constexpr (EPI == MM_SILU) X[(long long)m * ldc + n] = v * sigm(v);
+      }
     }
+  }
+  if constexpr (EPI == MM_PART) {
+    if (blockIdx.x == 0 && tid < BM && m0 + tid < M) C[((long long)blockIdx.z * M + m0 + tid) * (N + 1) + N] = csum;
   }
 }
 
-template <typename TB>
-void mm(int M, int N, int K, const float* A, int lda, int tA, const TB* B, int ldb, int tB, float* C, int ldc,
-        float alpha, float beta, const float* bias, float bias_scale, cudaStream_t st) {
+// 128-row tiles once they fill the chip (152 SMs), else 64-row ones (twice the blocks)
+template <typename TB, bool BT, int EPI>
+void mm(int M, int N, int K, const float* A, int lda, const TB* B, int ldb, float* C, int ldc, float alpha,
+        const float* bias, float* X, cudaStream_t st) {
   if (M <= 0 || N <= 0) return;
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
-  ++g_launch_count, k_mm<TB><<<grid, 256, 0, st>>>(M, N, K, A, lda, tA, B, ldb, tB, C, ldc, alpha, beta, bias,
-                                                   bias_scale);
+  const int nn = (N + 63) / 64;
+  if ((long long)nn * (M / 128) >= 152) {
+    ++g_launch_count, k_mm<128, TB, false, BT, EPI><<<dim3(nn, (M + 127) / 128), 256, 0, st>>>(M, N, K, K, A, lda, B, ldb,
+                                                                                             C, ldc, alpha, bias, X);
+  } else {
+    ++g_launch_count, k_mm<64, TB, false, BT, EPI><<<dim3(nn, (M + 63) / 64), 256, 0, st>>>(M, N, K, K, A, lda, B, ldb, C,
+                                                                                          ldc, alpha, bias, X);
+  }
+}
+
+// k parts of a gradient product: two blocks per SM, at least 256 rows each
+int grad_parts(int M, int N, int K) {
+  const int tiles = ((N + 63) / 64) * ((M + 127) / 128);
+  return std::max(1, std::min((2 * 152) / tiles, K / 256));
+}
+
+// gW[m][n] = alpha sum_z part[z][m][n], gb[m] (may be NULL) = alpha times column N
+__global__ void k_grad_sum(int M, int N, int parts, const float* __restrict__ part, float alpha, float* __restrict__ gW,
+                           float* __restrict__ gb) {
+  const long long n = (long long)M * (N + 1);
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    float v = 0.f;
+    for (int z = 0; z < parts; ++z) v += part[z * n + e];
+    const long long m = e / (N + 1);
+    const int c = (int)(e % (N + 1));
+    if (c < N) gW[m * N + c] = alpha * v;
+    else if (gb) gb[m] = alpha * v;
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
 // elementwise pieces
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ float sigm(float z) { return 1.f / (1.f + expf(-z)); }
-
-__global__ void k_silu_fwd(long long n, const float* __restrict__ Z, float* __restrict__ Hh) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float z = Z[i];
-    Hh[i] = z * sigm(z);
-  }
-}
-
-// dZ = dH * silu'(Z), silu'(z) = s (1 + z (1 - s)), s = sigmoid(z)
-__global__ void k_silu_bwd(long long n, const float* __restrict__ dH, const float* __restrict__ Z,
-                           float* __restrict__ dZ) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float z = Z[i], s = sigm(z);
-    dZ[i] = dH[i] * s * (1.f + z * (1.f - s));
-  }
-}
-
-// out[n] = alpha * sum_m A[m][n]  (one thread per column, rows in order)
-__global__ void k_colsum(int M, int N, const float* __restrict__ A, float alpha, float* __restrict__ out) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float acc = 0.f;
-  for (int m = 0; m < M; ++m) acc += A[(long long)m * N + n];
-  out[n] = alpha * acc;
-}
-
 // F = F + s G (F holds x L^T on entry); R = F - Y; dF = 2 R / (B n_out); loss += sum R^2 / (B n_out)
 __global__ void k_mse(long long n, float inv, float s, float* __restrict__ F, const float* __restrict__ G,
                       const float* __restrict__ Y, float* __restrict__ dF, double* __restrict__ loss) {
@@ -372,7 +423,7 @@ struct gw_surrogate_s {
   // activations for up to cap rows
   int cap = 0;
   float *xb = nullptr, *yb = nullptr, *Z1 = nullptr, *H1 = nullptr, *Z2 = nullptr, *H2 = nullptr, *Z3 = nullptr,
-        *H3 = nullptr, *G = nullptr, *F = nullptr, *dG = nullptr, *dA = nullptr, *dB = nullptr;
+        *H3 = nullptr, *G = nullptr, *F = nullptr, *dG = nullptr, *dA = nullptr, *dB = nullptr, *part = nullptr;
   std::vector<void*> allocs;
 };
 
@@ -403,7 +454,8 @@ void sfree(gw_surrogate_s* m, void* p) {
 
 gw_status ensure_cap(gw_surrogate_s* m, int rows) {
   if (rows <= m->cap) return GW_OK;
-  float** bufs[] = {&m->xb, &m->yb, &m->Z1, &m->H1, &m->Z2, &m->H2, &m->Z3, &m->H3, &m->G, &m->F, &m->dG, &m->dA, &m->dB};
+  float** bufs[] = {&m->xb, &m->yb, &m->Z1, &m->H1, &m->Z2, &m->H2, &m->Z3, &m->H3, &m->G, &m->F, &m->dG, &m->dA, &m->dB,
+                    &m->part};
   for (float** b : bufs) {
     sfree(m, *b);
     *b = nullptr;
@@ -423,45 +475,53 @@ gw_status ensure_cap(gw_surrogate_s* m, int rows) {
   MLP_TRY(salloc_n(m, &m->dG, r * wO));
   MLP_TRY(salloc_n(m, &m->dA, r * wH));
   MLP_TRY(salloc_n(m, &m->dB, r * wH));
+  // parts of the gradient products over up to `rows` rows
+  size_t parts = 0;
+  const int shapes[4][2] = {{m->O, m->H}, {m->H, m->H}, {m->H, m->I}, {m->O, m->I}};
+  for (const auto& s : shapes)
+    parts = std::max(parts, (size_t)grad_parts(s[0], s[1], rows) * s[0] * ((size_t)s[1] + 1));
+  MLP_TRY(salloc_n(m, &m->part, parts));
   m->cap = rows;
   return GW_OK;
 }
 
 // G = MLP(x) (without the output scale s) for B rows of x; activations kept for backward
 void forward_mlp(gw_surrogate_s* m, const float* x, int B, float* G, cudaStream_t st) {
+  using W = __nv_bfloat16;
   const int I = m->I, H = m->H, O = m->O;
   const Offs& o = m->off;
-  const long long nh = (long long)B * H;
-  mm<__nv_bfloat16>(B, H, I, x, I, 0, m->wb + o.W1, I, 1, m->Z1, H, 1.f, 0.f, m->th + o.b1, 1.f, st);
-  ++g_launch_count, k_silu_fwd<<<ew_grid(nh), 256, 0, st>>>(nh, m->Z1, m->H1);
-  mm<__nv_bfloat16>(B, H, H, m->H1, H, 0, m->wb + o.W2, H, 1, m->Z2, H, 1.f, 0.f, m->th + o.b2, 1.f, st);
-  ++g_launch_count, k_silu_fwd<<<ew_grid(nh), 256, 0, st>>>(nh, m->Z2, m->H2);
-  mm<__nv_bfloat16>(B, H, H, m->H2, H, 0, m->wb + o.W3, H, 1, m->Z3, H, 1.f, 0.f, m->th + o.b3, 1.f, st);
-  ++g_launch_count, k_silu_fwd<<<ew_grid(nh), 256, 0, st>>>(nh, m->Z3, m->H3);
-  mm<__nv_bfloat16>(B, O, H, m->H3, H, 0, m->wb + o.W4, H, 1, G, O, 1.f, 0.f, m->th + o.b4, 1.f, st);
+  mm<W, true, MM_SILU>(B, H, I, x, I, m->wb + o.W1, I, m->Z1, H, 1.f, m->th + o.b1, m->H1, st);
+  mm<W, true, MM_SILU>(B, H, H, m->H1, H, m->wb + o.W2, H, m->Z2, H, 1.f, m->th + o.b2, m->H2, st);
+  mm<W, true, MM_SILU>(B, H, H, m->H2, H, m->wb + o.W3, H, m->Z3, H, 1.f, m->th + o.b3, m->H3, st);
+  mm<W, true, MM_PLAIN>(B, O, H, m->H3, H, m->wb + o.W4, H, G, O, 1.f, m->th + o.b4, nullptr, st);
+}
+
+// gW[M][N] = alpha sum_r dZ[r][m] X[r][n], gb[m] = alpha sum_r dZ[r][m] over the B rows
+void weight_grad(gw_surrogate_s* m, int M, int N, int B, const float* dZ, const float* X, float alpha, float* gW,
+                 float* gb, cudaStream_t st) {
+  const int parts = grad_parts(M, N, B), kpart = ((B + parts - 1) / parts + 15) / 16 * 16;
+  const int used = (B + kpart - 1) / kpart;
+  ++g_launch_count, k_mm<128, float, true, false, MM_PART><<<dim3((N + 63) / 64, (M + 127) / 128, used), 256, 0, st>>>(
+      M, N, B, kpart, dZ, M, X, N, m->part, 0, 1.f, nullptr, nullptr);
+  const long long n = (long long)M * (N + 1);
+  ++g_launch_count, k_grad_sum<<<(int)std::min<long long>((n + 255) / 256, 152LL * 16), 256, 0, st>>>(M, N, used, m->part,
+                                                                                                    alpha, gW, gb);
 }
 
 // gradients of the W/b parameters from dG = dLoss/d(MLP output) for the B rows of x (alpha
 // scales every gradient, e.g. by s); fills m->grad[W1 .. b4]
 void backward_mlp(gw_surrogate_s* m, const float* x, int B, const float* dG, float alpha, cudaStream_t st) {
+  using W = __nv_bfloat16;
   const int I = m->I, H = m->H, O = m->O;
   const Offs& o = m->off;
-  const long long nh = (long long)B * H;
   float* g = m->grad;
-  mm<float>(O, H, B, dG, O, 1, m->H3, H, 0, g + o.W4, H, alpha, 0.f, nullptr, 0.f, st);
-  ++g_launch_count, k_colsum<<<(O + 127) / 128, 128, 0, st>>>(B, O, dG, alpha, g + o.b4);
-  mm<__nv_bfloat16>(B, H, O, dG, O, 0, m->wb + o.W4, H, 0, m->dA, H, alpha, 0.f, nullptr, 0.f, st);
-  ++g_launch_count, k_silu_bwd<<<ew_grid(nh), 256, 0, st>>>(nh, m->dA, m->Z3, m->dB);  // dZ3
-  mm<float>(H, H, B, m->dB, H, 1, m->H2, H, 0, g + o.W3, H, 1.f, 0.f, nullptr, 0.f, st);
-  ++g_launch_count, k_colsum<<<(H + 127) / 128, 128, 0, st>>>(B, H, m->dB, 1.f, g + o.b3);
-  mm<__nv_bfloat16>(B, H, H, m->dB, H, 0, m->wb + o.W3, H, 0, m->dA, H, 1.f, 0.f, nullptr, 0.f, st);
-  ++g_launch_count, k_silu_bwd<<<ew_grid(nh), 256, 0, st>>>(nh, m->dA, m->Z2, m->dB);  // dZ2
-  mm<float>(H, H, B, m->dB, H, 1, m->H1, H, 0, g + o.W2, H, 1.f, 0.f, nullptr, 0.f, st);
-  ++g_launch_count, k_colsum<<<(H + 127) / 128, 128, 0, st>>>(B, H, m->dB, 1.f, g + o.b2);
-  mm<__nv_bfloat16>(B, H, H, m->dB, H, 0, m->wb + o.W2, H, 0, m->dA, H, 1.f, 0.f, nullptr, 0.f, st);
-  ++g_launch_count, k_silu_bwd<<<ew_grid(nh), 256, 0, st>>>(nh, m->dA, m->Z1, m->dB);  // dZ1
-  mm<float>(H, I, B, m->dB, H, 1, x, I, 0, g + o.W1, I, 1.f, 0.f, nullptr, 0.f, st);
-  ++g_launch_count, k_colsum<<<(H + 127) / 128, 128, 0, st>>>(B, H, m->dB, 1.f, g + o.b1);
+  weight_grad(m, O, H, B, dG, m->H3, alpha, g + o.W4, g + o.b4, st);
+  mm<W, false, MM_DSILU>(B, H, O, dG, O, m->wb + o.W4, H, m->dA, H, alpha, nullptr, m->Z3, st);    // dZ3
+  weight_grad(m, H, H, B, m->dA, m->H2, 1.f, g + o.W3, g + o.b3, st);
+  mm<W, false, MM_DSILU>(B, H, H, m->dA, H, m->wb + o.W3, H, m->dB, H, 1.f, nullptr, m->Z2, st);   // dZ2
+  weight_grad(m, H, H, B, m->dB, m->H1, 1.f, g + o.W2, g + o.b2, st);
+  mm<W, false, MM_DSILU>(B, H, H, m->dB, H, m->wb + o.W2, H, m->dA, H, 1.f, nullptr, m->Z1, st);   // dZ1
+  weight_grad(m, H, I, B, m->dA, x, 1.f, g + o.W1, g + o.b1, st);
 }
 
 gw_status begin(gw_surrogate_s* m) {
@@ -617,7 +677,7 @@ gw_status gw_surrogate_forward(gw_surrogate m, const float* x, int64_t n, float*
     if (g) ++g_launch_count, k_scale_copy<<<ew_grid(no), 256, 0, m->st>>>(no, m->h_s, m->G, g + r0 * O);
     if (f) {
       float* fr = f + r0 * O;
-      mm<float>(B, O, I, xr, I, 0, m->th + m->off.L, I, 1, fr, O, 1.f, 0.f, nullptr, 0.f, m->st);
+      mm<float, true, MM_PLAIN>(B, O, I, xr, I, m->th + m->off.L, I, fr, O, 1.f, nullptr, nullptr, m->st);
       ++g_launch_count, k_mse<<<ew_grid(no), 256, 0, m->st>>>(no, 0.f, m->h_s, fr, m->G, nullptr, nullptr, nullptr);
     }
   }
@@ -634,12 +694,12 @@ gw_status gw_surrogate_loss_grad(gw_surrogate m, const float* x, const float* y,
   MLP_TRY(ensure_cap(m, B));
   MLP_CUDA(cudaMemsetAsync(m->d_acc, 0, sizeof(double), m->st));
   forward_mlp(m, x, B, m->G, m->st);
-  mm<float>(B, O, I, x, I, 0, m->th + o.L, I, 1, m->F, O, 1.f, 0.f, nullptr, 0.f, m->st);
+  mm<float, true, MM_PLAIN>(B, O, I, x, I, m->th + o.L, I, m->F, O, 1.f, nullptr, nullptr, m->st);
   const long long no = (long long)B * O;
   ++g_launch_count, k_mse<<<ew_grid(no), 256, 0, m->st>>>(no, 1.f / (float)no, m->h_s, m->F, m->G, y, m->dG,
                                                           m->d_acc);
   backward_mlp(m, x, B, m->dG, m->h_s, m->st);
-  mm<float>(O, I, B, m->dG, O, 1, x, I, 0, m->grad + o.L, I, 1.f, 0.f, nullptr, 0.f, m->st);
+  weight_grad(m, O, I, B, m->dG, x, 1.f, m->grad + o.L, nullptr, m->st);
   MLP_CUDA(cudaMemsetAsync(m->grad + o.s, 0, sizeof(float), m->st));
   MLP_CUDA(cudaMemcpyAsync(grad, m->grad, (size_t)o.P * sizeof(float), cudaMemcpyDeviceToDevice, m->st));
   double h = 0.0;
