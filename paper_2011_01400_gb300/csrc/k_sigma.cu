@@ -32,69 +32,86 @@ template void launch_rowdot<float>(int, int, const c64*, const c64*, long long, 
                                    cudaStream_t);
 
 // sigma[k][n][w] += pref * sum_m sum_j g_j S[(kk,n,m)][j] 2 z / (z^2 + w_j^2),  z = i w + mu - eps_m(k - q)
-// Rows of S are r = ((kk * nsig) + n) * NBd + m for k = kk0 + kk. One thread per (kk, n, w).
+// Rows of S are r = ((kk * nsig) + n) * NBd + m for k = kk0 + kk. One block per (kk, n): thread
+// (part, w) sums the bands m = part, part + parts, ... for one output frequency, the parts are added in
+// order in FP64. A kernel value (a division and ~15 FMAs) per (m, j, w) bounds it; S is read by whole
+// warps at one address. 216 k, 8 window bands, 78 bands, 32 frequencies: 140 us, 487 us with one thread
+// per (kk, n, w); one k, 300 bands, where that filled two blocks: 48 us, 1254 us before.
 template <typename T>
-__global__ void k_sigma_conv(int nkk, int kk0, int nsig, int NBd, int n1, int n2, int n3, int q,
-                             const double* __restrict__ eps, const double* __restrict__ mu_p,
-                             const float* __restrict__ S_f, const double* __restrict__ S_d,
-                             const double* __restrict__ freq, const double* __restrict__ gw, int nw, double pref,
-                             c128* __restrict__ sigma, const int* __restrict__ ktab) {
+__global__ void k_sigma_conv(int kk0, int nsig, int NBd, int n1, int n2, int n3, int q, const double* __restrict__ eps,
+                             const double* __restrict__ mu_p, const float* __restrict__ S_f,
+                             const double* __restrict__ S_d, const double* __restrict__ freq,
+                             const double* __restrict__ gw, int nw, double pref, c128* __restrict__ sigma,
+                             const int* __restrict__ ktab) {
   extern __shared__ double sh[];
-  double* fr = sh;
-  double* gg = sh + nw;
+  double2* red = reinterpret_cast<double2*>(sh);           // [parts * nw]
+  T* fr2 = reinterpret_cast<T*>(sh + 2 * blockDim.x);      // w_j^2
+  T* gg = fr2 + nw;
   for (int i = threadIdx.x; i < nw; i += blockDim.x) {
-    fr[i] = freq[i];
-    gg[i] = gw[i];
+    const T w = (T)freq[i];
+    fr2[i] = w * w;
+    gg[i] = (T)gw[i];
   }
   __syncthreads();
-  const int total = nkk * nsig * nw;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= total) return;
-  const int w_i = t % nw, n = (t / nw) % nsig, kk = t / (nw * nsig);
+  const int n = blockIdx.x % nsig, kk = blockIdx.x / nsig;
+  const int w_i = threadIdx.x % nw, part = threadIdx.x / nw, parts = blockDim.x / nw;
   const int k = ktab ? ktab[kk0 + kk] : kk0 + kk;
-  int k3 = k % n3, k2 = (k / n3) % n2, k1 = k / (n2 * n3);
-  int q3 = q % n3, q2 = (q / n3) % n2, q1 = q / (n2 * n3);
-  int kmq = (((k1 - q1 + n1) % n1) * n2 + ((k2 - q2 + n2) % n2)) * n3 + ((k3 - q3 + n3) % n3);
-  const T om = (T)fr[w_i];
-  const T mu = (T)*mu_p;
-  T acc_re = 0, acc_im = 0;
-  for (int m = 0; m < NBd; ++m) {
-    const long long r = ((long long)kk * nsig + n) * NBd + m;
-    const T zr = mu - (T)eps[(long long)kmq * NBd + m];   // z = zr + i om
-    // z^2 = zr^2 - om^2 + 2 i zr om
-    const T z2r = zr * zr - om * om, z2i = (T)2 * zr * om;
-    T sr = 0, si = 0;
-    for (int j = 0; j < nw; ++j) {
-      const T s = (T)gg[j] * (S_d ? (T)S_d[r * nw + j] : (T)S_f[r * nw + j]);
-      const T wj = (T)fr[j];
-      // 2 z / (z^2 + wj^2)
-      const T dr = z2r + wj * wj, di = z2i;
-      const T inv = (T)1 / (dr * dr + di * di);
-      const T fr_ = (T)2 * (zr * dr + om * di) * inv;
-      const T fi_ = (T)2 * (om * dr - zr * di) * inv;
-      sr += s * fr_;
-      si += s * fi_;
+  const int k3 = k % n3, k2 = (k / n3) % n2, k1 = k / (n2 * n3);
+  const int q3 = q % n3, q2 = (q / n3) % n2, q1 = q / (n2 * n3);
+  const int kmq = (((k1 - q1 + n1) % n1) * n2 + ((k2 - q2 + n2) % n2)) * n3 + ((k3 - q3 + n3) % n3);
+  if (part < parts) {
+    const T om = (T)freq[w_i];
+    const T mu = (T)*mu_p;
+    T acc_re = 0, acc_im = 0;
+    for (int m = part; m < NBd; m += parts) {
+      const long long r = ((long long)kk * nsig + n) * NBd + m;
+      const T zr = mu - (T)eps[(long long)kmq * NBd + m];   // z = zr + i om
+      // z^2 = zr^2 - om^2 + 2 i zr om
+      const T z2r = zr * zr - om * om, di = (T)2 * zr * om;
+      T sr = 0, si = 0;
+#pragma unroll 4
+      for (int j = 0; j < nw; ++j) {
+        const T s = gg[j] * (S_d ? (T)S_d[r * nw + j] : (T)S_f[r * nw + j]);
+        // 2 z / (z^2 + wj^2)
+        const T dr = z2r + fr2[j];
+        const T inv = (T)1 / (dr * dr + di * di);
+        const T fr_ = (T)2 * (zr * dr + om * di) * inv;
+        const T fi_ = (T)2 * (om * dr - zr * di) * inv;
+        sr += s * fr_;
+        si += s * fi_;
+      }
+      acc_re += sr;
+      acc_im += si;
     }
-    acc_re += sr;
-    acc_im += si;
+    red[threadIdx.x] = make_double2((double)acc_re, (double)acc_im);
   }
-  c128* o = sigma + ((long long)k * nsig + n) * nw + w_i;
-  o->re += pref * (double)acc_re;
-  o->im += pref * (double)acc_im;
+  __syncthreads();
+  if (threadIdx.x < nw) {
+    double re = 0.0, im = 0.0;
+    for (int p = 0; p < parts; ++p) {
+      const double2 v = red[p * nw + threadIdx.x];
+      re += v.x;
+      im += v.y;
+    }
+    c128* o = sigma + ((long long)k * nsig + n) * nw + threadIdx.x;
+    o->re += pref * re;
+    o->im += pref * im;
+  }
 }
 
 void launch_sigma_conv_chunk(int kk0, int nkk, int nsig, int NBd, const int* nk, int q, const double* eps,
                              const double* mu, const float* S_f, const double* S_d, const double* freq,
                              const double* gw, int nw, double pref, c128* sigma, bool fp64, cudaStream_t st,
                              const int* ktab) {
-  int total = nkk * nsig * nw;
-  size_t smem = 2 * nw * sizeof(double);
+  // few (k, n): more bands side by side in a block (the FP64 kernel keeps to 512 threads' registers)
+  const int nt = nkk * nsig >= 304 ? 256 : (fp64 ? 512 : 1024);
+  const size_t smem = 2 * sizeof(double) * nt + 2 * sizeof(double) * nw;
   if (fp64)
-    ++::gw::g_launch_count, k_sigma_conv<double><<<(total + 127) / 128, 128, smem, st>>>(nkk, kk0, nsig, NBd, nk[0], nk[1], nk[2], q, eps,
-                                                                 mu, S_f, S_d, freq, gw, nw, pref, sigma, ktab);
+    ++::gw::g_launch_count, k_sigma_conv<double><<<nkk * nsig, nt, smem, st>>>(kk0, nsig, NBd, nk[0], nk[1], nk[2], q, eps, mu, S_f,
+                                                                              S_d, freq, gw, nw, pref, sigma, ktab);
   else
-    ++::gw::g_launch_count, k_sigma_conv<float><<<(total + 127) / 128, 128, smem, st>>>(nkk, kk0, nsig, NBd, nk[0], nk[1], nk[2], q, eps,
-                                                                mu, S_f, S_d, freq, gw, nw, pref, sigma, ktab);
+    ++::gw::g_launch_count, k_sigma_conv<float><<<nkk * nsig, nt, smem, st>>>(kk0, nsig, NBd, nk[0], nk[1], nk[2], q, eps, mu, S_f,
+                                                                             S_d, freq, gw, nw, pref, sigma, ktab);
 }
 
 __global__ void k_sigma_trs_fill(int NK, int nsig, int nw, int n1, int n2, int n3, const int* __restrict__ is_rep,
