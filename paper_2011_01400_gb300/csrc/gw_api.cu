@@ -1148,7 +1148,9 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
   const int N = P->N, nw = P->nw;
   const size_t NN = (size_t)N * N;
   const c128* evec = reinterpret_cast<const c128*>(P->p.evec);
-  GW_CUDA(cudaMemsetAsync(chi0, 0, sizeof(c128) * NN * nw, st));
+  // frequency compression (split precision): chi0(w_j) = sum_t U_jt C_t over T <= nw weight rows
+  const bool comp = compress_on(P);
+  if (!comp) GW_CUDA(cudaMemsetAsync(chi0, 0, sizeof(c128) * NN * nw, st));
   const bool hw = P->p.head_wings && q == 0;
   const bool hw_avg = hw && P->p.head_wings == 2;
   if (hw) {
@@ -1172,8 +1174,6 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
   const double hw_pref = 4.0 * M_PI * P->p.spin / (P->p.omega_cell * P->NK);
   const double scale = -P->p.spin / P->NK;
   const int na = P->nunocc, nb = P->nocc;
-  // frequency compression (split precision): chi0(w_j) = sum_t U_jt C_t over T <= nw weight rows
-  const bool comp = compress_on(P);
   int jq = 0;                 // position of q in the list of prepared weight bases
   int T = nw;
   const double* Uw = nullptr;
@@ -1279,8 +1279,8 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
     }
     GW_TRY(check_launch(P, "chi0"));
   }
-  if (comp) launch_expand(nw, T, (long long)NN, Uw, P->d_C, chi0, st);
-  if (!P->fp64) tc_herm_fill(N, nw, chi0, st);
+  if (comp) launch_expand(N, nw, T, Uw, P->d_C, chi0, st);
+  else if (!P->fp64) tc_herm_fill(N, nw, chi0, st);
   P->chi0_flops_acc += 8.0 * (double)P->NK * na * nb * ((double)N * (N + 1) / 2) * nw;
   return GW_OK;
 }

@@ -240,7 +240,7 @@ void launch_wresid(int K, int nw, const double* delta, const double* freq, const
                    double* err, cudaStream_t st);
 void launch_wtab_compressed(int K, int Kpad, int nw, int T, const double* delta, const double* freq, const double* Pm,
                             float* wtab, cudaStream_t st);
-void launch_expand(int nw, int T, long long NN, const double* E, const c128* C, c128* chi0, cudaStream_t st);
+void launch_expand(int N, int nw, int T, const double* E, const c128* C, c128* chi0, cudaStream_t st);
 
 // text returned by gw_last_error() on this thread
 void gw_set_last_error(const std::string& msg);
