@@ -35,11 +35,6 @@
  *     GW_WORKSPACE_LIMIT    bytes of device memory one plan may allocate for its workspace
  *                           (default: no limit). An allocation that would pass it fails with
  *                           GW_ERR_NOMEM before cudaMalloc is called.
- *   - Autotuning: the first split-precision call that generates band-pair rows
- *     of a given shape in this process times two thread mappings of that kernel
- *     (one warm-up and one timed launch each). It then waits for the plan's stream
- *     once, to read the timings. Both mappings write identical rows, so the
- *     results never depend on the choice, and later calls of that shape do not wait.
  */
 #ifndef GW_H
 #define GW_H

@@ -2,12 +2,10 @@
 #include "gw_internal.h"
 
 #include <algorithm>
-#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <map>
 #include <mutex>
 #include <new>
 #include <string>
@@ -190,56 +188,6 @@ struct SurState {
   float *d_d = nullptr, *d_x = nullptr, *d_sig = nullptr, *d_g = nullptr, *d_coef = nullptr;
 };
 
-// Autotuner of the fp32 shared-memory M kernels. Per device and call shape (kernel, na, nb) both
-// thread mappings are run at first use on the calling plan's stream -- one warm-up launch, then one
-// timed launch each (CUDA events) -- and the faster one is recorded process-wide for every later
-// call of that shape. The two mappings write bit-identical rows, so the repeated launches only cost
-// time; results never depend on the choice.
-struct MgenTuner {
-  cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
-  static std::map<std::array<int, 4>, int>& table() {
-    static std::map<std::array<int, 4>, int> t;
-    return t;
-  }
-  static std::mutex& table_mutex() {
-    static std::mutex m;
-    return m;
-  }
-  ~MgenTuner() {
-    for (cudaEvent_t e : ev)
-      if (e) cudaEventDestroy(e);
-  }
-  // launch(variant) issues the kernel on st; returns false on a CUDA error
-  template <typename F> bool run(int kind, int na, int nb, cudaStream_t st, F&& launch) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    const std::array<int, 4> key{dev, kind, na, nb};
-    {
-      std::lock_guard<std::mutex> lk(table_mutex());
-      auto it = table().find(key);
-      if (it != table().end()) {
-        const int v = it->second;
-        launch(v);
-        return true;
-      }
-    }
-    for (cudaEvent_t& e : ev)
-      if (!e && cudaEventCreate(&e) != cudaSuccess) return false;
-    launch(0);
-    if (cudaEventRecord(ev[0], st) != cudaSuccess) return false;
-    launch(0);
-    if (cudaEventRecord(ev[1], st) != cudaSuccess) return false;
-    launch(1);
-    if (cudaEventRecord(ev[2], st) != cudaSuccess || cudaEventSynchronize(ev[2]) != cudaSuccess) return false;
-    float t0 = 0.f, t1 = 0.f;
-    if (cudaEventElapsedTime(&t0, ev[0], ev[1]) != cudaSuccess || cudaEventElapsedTime(&t1, ev[1], ev[2]) != cudaSuccess)
-      return false;
-    std::lock_guard<std::mutex> lk(table_mutex());
-    table()[key] = (t1 < t0) ? 1 : 0;
-    return true;
-  }
-};
-
 struct gw_plan_s {
   gw_problem p{};
   gw_precision prec;
@@ -290,7 +238,8 @@ struct gw_plan_s {
   int* d_status = nullptr;
   // chunk workspaces
   int chi_nkk = 1, sig_nkk = 1;
-  void* d_M = nullptr;        // chi0 M [N][ldm] (c128 or c64)
+  c64* d_evec32 = nullptr;    // split precision: FP32 copy of the eigenvectors [NK][NB][NBd]
+  c128* d_M = nullptr;        // FP64: chi0 M [N][ldm]
   long long ldm = 0;
   double* d_delta = nullptr;  // [ldm]
   float* d_delta_f = nullptr;
@@ -338,7 +287,6 @@ struct gw_plan_s {
   uint8_t* g_work = nullptr;
   int qb = 0;
   double group_budget = 8.0e9;  // bytes for the q-group buffers of gw_g0w0
-  MgenTuner mtune;              // picks the thread mapping of the fp32 M kernels per call shape
   SurState sur;
   // batch plan (n_sys > 1): one plan per system, each on its own stream; the batch plan itself
   // holds no device memory
@@ -838,11 +786,10 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
     P->d_U = c;
     ALLOC(P->d_S_d, (size_t)P->sig_rows * nw);
   } else {
-    c64 *a, *b;
+    c64* b;
     P->Kx = ((N + 31) / 32) * 32;
-    ALLOC(a, (size_t)N * P->ldm);
+    ALLOC(P->d_evec32, (size_t)P->NK * P->NB * P->NBd);
     ALLOC(b, (size_t)P->sig_rows * P->Kx);   // raw plane of the Sigma rows, zero beyond n_aux
-    P->d_M = a;
     P->d_A = b;
     ALLOC(P->d_S_f, (size_t)P->sig_rows * nw);
     for (int i = 0; i < 2; ++i) {
@@ -1015,8 +962,9 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
     launch_rank1(N, P->d_Vh, P->d_x1, std::sqrt(std::max(P->h_v1, 0.0)), st);
   }
   if (!P->fp64) {
-    launch_convert((int)(NN * P->NK), P->d_Vh, P->d_Vh32, st);
-    if (prob->head_wings) launch_convert((int)NN, P->d_Vb0, P->d_Vb32, st);
+    launch_convert((long long)P->NK * P->NB * P->NBd, reinterpret_cast<const c128*>(prob->evec), P->d_evec32, st);
+    launch_convert((long long)NN * P->NK, P->d_Vh, P->d_Vh32, st);
+    if (prob->head_wings) launch_convert((long long)NN, P->d_Vb0, P->d_Vb32, st);
     CK(cudaMemsetAsync(P->d_A, 0, sizeof(c64) * (size_t)P->sig_rows * P->Kx, st));
   }
   if ((s = check_launch(P, "plan setup")) != GW_OK) return cleanup(s);
@@ -1197,8 +1145,8 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
                  reinterpret_cast<const c128*>(P->p.pmom), P->p.qhat, P->d_delta, P->d_delta_f,
                  hw ? P->d_pq : nullptr, st);
     if (P->fp64) {
-      c128* M = static_cast<c128*>(P->d_M);
-      launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), nullptr, evec, q, kk0, nkk, MAP_K_IS_KK,
+      c128* M = P->d_M;
+      launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), evec, q, kk0, nkk, MAP_K_IS_KK,
                           P->nocc, na, 0, nb, M, 1, P->ldm, st);
       GW_CUDA(cudaEventRecord(e0, st));
       launch_chi0_simt<double>(N, K, M, P->ldm, nullptr, P->d_delta, P->d_freq, nw, scale, chi0, st);
@@ -1224,13 +1172,8 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
         GW_CUDA(cudaMemsetAsync(P->d_delta_f + K, 0, sizeof(float) * (P->ldm - K), st));
       }
       GW_CUDA(cudaMemsetAsync(P->d_absmax, 0, sizeof(unsigned), st));
-      if (!launch_mgen_chi(P->geom, static_cast<const c64*>(P->d_T1), evec, q, kk0, nkk, P->nocc, na, 0, nb,
-                           P->d_Praw, 2 * P->ldm, 0, P->d_absmax, st) &&
-          !P->mtune.run(1, na, nb, st, [&](int v) {
-            launch_mgen_planes(P->geom, static_cast<const c64*>(P->d_T1), evec, q, kk0, nkk, P->nocc, na, 0, nb,
-                               P->d_Praw, nullptr, 2 * P->ldm, 0, 0, st, v, P->d_absmax);
-          }))
-        return fail(GW_ERR_CUDA, "M kernel autotuner: CUDA error");
+      launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), P->d_evec32, q, kk0, nkk, MAP_K_IS_KK, P->nocc, na, 0,
+                         nb, reinterpret_cast<c64*>(P->d_Praw), 1, P->ldm, st, P->d_absmax);
       Chi0hArgs a{};
       a.kind = kind;
       a.N = N;
@@ -1261,12 +1204,7 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
         return fail(ts, err);
       }
       if (hw) {
-        c64* M = static_cast<c64*>(P->d_M);
-        if (!P->mtune.run(0, na, nb, st, [&](int v) {
-              launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), nullptr, evec, q, kk0, nkk, MAP_K_IS_KK,
-                                 P->nocc, na, 0, nb, M, 1, P->ldm, st, v);
-            }))
-          return fail(GW_ERR_CUDA, "M kernel autotuner: CUDA error");
+        const c64* M = reinterpret_cast<const c64*>(P->d_Praw);
         if (!hw_avg)
           launch_head_wings<float>(N, K, M, P->ldm, P->d_delta, P->d_pq, P->d_freq, nw, hw_pref, P->d_head, P->d_h,
                                    st);
@@ -1346,7 +1284,7 @@ gw_status eps_core(gw_plan_s* P, int q, const c128* chi0, c128* E) {
     const c64* Vh32 = P->d_Vh32 + (long long)q * NN;
     const c64* Vin32 = hw ? P->d_Vb32 : Vh32;
     GW_TRY(herm_gemm(P, Vin32, false, chi0, true, 1.0, P->d_tmp));
-    launch_convert((int)(NN * nw), P->d_tmp, A32, st);
+    launch_convert(NN * nw, P->d_tmp, A32, st);
     GW_TRY(herm_gemm(P, A32, true, Vin, false, -1.0, E));
   }
   launch_axpby_identity<double>(N, E, NN, nw, 1.0, st);
@@ -1396,7 +1334,7 @@ gw_status w_core(gw_plan_s* P, int q, const c128* X, c128* Wc) {
     // V^1/2 X V^1/2 as (V^1/2 X) V^1/2 (X = eps~^-1 - 1 and V^1/2 Hermitian)
     const c64* Vh32 = P->d_Vh32 + (long long)q * NN;
     GW_TRY(herm_gemm(P, Vh32, false, X, true, 1.0, P->d_tmp));
-    launch_convert((int)(NN * nw), P->d_tmp, A32, st);
+    launch_convert(NN * nw, P->d_tmp, A32, st);
     GW_TRY(herm_gemm(P, A32, true, Vh, false, 1.0, Wc));
   }
   return check_launch(P, "W^c");
@@ -1424,7 +1362,7 @@ gw_status sigma_core(gw_plan_s* P, int q, const c128* Wc, c128* sig, bool conjW 
     if (P->fp64) {
       c128* A = static_cast<c128*>(P->d_A);
       c128* U = static_cast<c128*>(P->d_U);
-      launch_mgen<double>(geom, static_cast<const c128*>(P->d_T1), nullptr, evec, q, kk0, nkk,
+      launch_mgen<double>(geom, static_cast<const c128*>(P->d_T1), evec, q, kk0, nkk,
                           MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, NBd, A, N, 1, st);
       for (int j = 0; j < nw; ++j) {
         launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, Wc + j * NN, N, 0, conjW ? OP_CONJ : OP_N,
@@ -1434,13 +1372,8 @@ gw_status sigma_core(gw_plan_s* P, int q, const c128* Wc, c128* sig, bool conjW 
     } else {
       // rows a_r as an fp32 plane [R][Kx] (zero beyond n_aux), then the tensor-core contraction
       c64* A = static_cast<c64*>(P->d_A);
-      if (!launch_mgen_sig(geom, static_cast<const c64*>(P->d_T1), evec, q, kk0, nkk, P->p.sigma_lo, nsig, NBd, A,
-                           P->Kx, 1, st) &&
-          !P->mtune.run(0, nsig, NBd, st, [&](int v) {
-            launch_mgen<float>(geom, static_cast<const c64*>(P->d_T1), nullptr, evec, q, kk0, nkk,
-                               MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, NBd, A, P->Kx, 1, st, v);
-          }))
-        return fail(GW_ERR_CUDA, "M kernel autotuner: CUDA error");
+      launch_mgen<float>(geom, static_cast<const c64*>(P->d_T1), P->d_evec32, q, kk0, nkk, MAP_K_IS_KK_MINUS_Q,
+                         P->p.sigma_lo, nsig, 0, NBd, A, P->Kx, 1, st);
       GW_CUDA(cudaMemsetAsync(P->d_S_f, 0, sizeof(float) * (size_t)R * nw, st));
       TcSigmaArgs a{};
       a.R = R;
@@ -1920,7 +1853,7 @@ gw_status sigma_core_sur(gw_plan_s* P, int q, const c128* Wc_c, const c128* U, c
     if (P->fp64) {
       c128* A = static_cast<c128*>(P->d_A);
       c128* Ut = static_cast<c128*>(P->d_U);
-      launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), nullptr, evec, q, kk0, nkk,
+      launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), evec, q, kk0, nkk,
                           MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, NBd, A, N, 1, st);
       for (int c = 0; c < nc; ++c) {
         launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, Wc_c + c * NN, N, 0, OP_N, c128{0, 0}, Ut, N, 0, 1, st);
@@ -1931,13 +1864,8 @@ gw_status sigma_core_sur(gw_plan_s* P, int q, const c128* Wc_c, const c128* U, c
       launch_sur_assemble<double>(R, nc, nw, k, S.d_jmap, S.d_Sc_d, Pm, coef, nf, Lmat, P->d_S_d, st);
     } else {
       c64* A = static_cast<c64*>(P->d_A);
-      if (!launch_mgen_sig(P->geom, static_cast<const c64*>(P->d_T1), evec, q, kk0, nkk, P->p.sigma_lo, nsig, NBd,
-                           A, P->Kx, 1, st) &&
-          !P->mtune.run(0, nsig, NBd, st, [&](int v) {
-            launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), nullptr, evec, q, kk0, nkk,
-                               MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, NBd, A, P->Kx, 1, st, v);
-          }))
-        return fail(GW_ERR_CUDA, "M kernel autotuner: CUDA error");
+      launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), P->d_evec32, q, kk0, nkk, MAP_K_IS_KK_MINUS_Q,
+                         P->p.sigma_lo, nsig, 0, NBd, A, P->Kx, 1, st);
       GW_CUDA(cudaMemsetAsync(S.d_Sc, 0, sizeof(float) * (size_t)R * nc, st));
       TcSigmaArgs a{};
       a.R = R;
@@ -2277,24 +2205,21 @@ gw_status gw_sigma_x(gw_plan P, int32_t sys, double* sigx) {
   const c128* V = reinterpret_cast<const c128*>(P->p.V);
   GW_CUDA(cudaMemsetAsync(sigx, 0, sizeof(double) * P->NK * nsig, st));
   for (int q = 0; q < P->NK; ++q) {
-    if (!P->fp64) launch_convert((int)NN, V + q * NN, P->d_Vx32, st);
+    if (!P->fp64) launch_convert((long long)NN, V + q * NN, P->d_Vx32, st);
     for (int kk0 = 0; kk0 < P->NK; kk0 += P->sig_nkk) {
       const int nkk = std::min(P->sig_nkk, P->NK - kk0);
       const int R = nkk * nsig * nocc;
       if (P->fp64) {
         c128* A = static_cast<c128*>(P->d_A);
         c128* U = static_cast<c128*>(P->d_U);
-        launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), nullptr, evec, q, kk0, nkk,
+        launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), evec, q, kk0, nkk,
                             MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, nocc, A, N, 1, st);
         launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, V + q * NN, N, 0, OP_N, c128{0, 0}, U, N, 0, 1, st);
         launch_rowdot<double>(R, N, U, A, N, nullptr, P->d_Sx, 0, 1, st);
       } else {
         c64* A = static_cast<c64*>(P->d_A);
-        if (!P->mtune.run(0, nsig, nocc, st, [&](int v) {
-              launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), nullptr, evec, q, kk0, nkk,
-                                 MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, nocc, A, P->Kx, 1, st, v);
-            }))
-          return fail(GW_ERR_CUDA, "M kernel autotuner: CUDA error");
+        launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), P->d_evec32, q, kk0, nkk, MAP_K_IS_KK_MINUS_Q,
+                           P->p.sigma_lo, nsig, 0, nocc, A, P->Kx, 1, st);
         launch_zgemm<float>(R, N, N, c64{1, 0}, A, P->Kx, 0, OP_N, P->d_Vx32, N, 0, OP_N, c64{0, 0}, P->d_Ux, P->Kx,
                             0, 1, st);
         launch_rowdot<float>(R, N, P->d_Ux, A, P->Kx, nullptr, P->d_Sx, 0, 1, st);

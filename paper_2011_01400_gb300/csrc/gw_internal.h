@@ -68,28 +68,13 @@ void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, cp
 // M^mu_{ab}(k', q) for a in [a0, a0+na) at k'+q and b in [b0, b0+nb) at k', for the k' of each row block.
 // Row index r = ((kk * na) + a) * nb + b for kk in [0, nkk); k' = kmap(kk) (see MapMode).
 // out element (r, mu) at out[r * s_r + mu * s_mu].
-// variant (fp32 shared-memory kernels): thread mapping, 0 = one output per thread, 1 = one (a, b)
-// pair per thread over the tile's ABFs; both give bit-identical rows (picked by MgenTuner).
+// absmax (fp32 only, may be NULL) receives max |re|, |im| of the rows written, as float bits
+// (atomicMax; the caller zeroes it). evec: the eigenvectors in the precision of the rows.
 enum MapMode { MAP_K_IS_KK = 0, MAP_K_IS_KK_MINUS_Q = 1 };
 template <typename T>
-void launch_mgen(const LriGeom& g, const cplx<T>* T1, const cplx<T>* T2, const c128* evec, int q,
-                 int kk0, int nkk, MapMode mode, int a0, int na, int b0, int nb, cplx<T>* out, long long s_r,
-                 long long s_mu, cudaStream_t st, int variant = 0);
-// Sigma_c rows of the split path, streamed (window of at most 8 bands, n_b(A) <= 48); returns
-// false when the shape is outside that range (the caller then uses launch_mgen<float>)
-bool launch_mgen_sig(const LriGeom& g, const c64* T1, const c128* evec, int q, int kk0, int nkk, int a0, int na,
-                     int nb, c64* out, long long s_r, long long s_mu, cudaStream_t st);
-// chi0 pair rows of the split path as the fp32 plane (streamed; at most 8 occupied bands,
-// n_b(A) <= 48), largest |re|, |im| into absmax; false outside that range
-bool launch_mgen_chi(const LriGeom& g, const c64* T1, const c128* evec, int q, int kk0, int nkk, int a0, int na,
-                     int b0, int nb, float* raw, long long ldk, long long kofs, unsigned* absmax, cudaStream_t st);
-// split planes for the tensor-core chi0 B operand: for row mu, K index 2r + {0: re, 1: im}
-// raw fp32 plane + B1/B2 split planes (3 BF16 pieces or 2 TF32 pieces each), see k_lri.cu
-// bplanes may be NULL (raw plane only); absmax (may be NULL) receives max |re|, |im| of the rows
-// written, as float bits (atomicMax; the caller zeroes it)
-void launch_mgen_planes(const LriGeom& g, const c64* T1, const c128* evec, int q, int kk0, int nkk, int a0, int na,
-                        int b0, int nb, float* raw, void* const* bplanes, long long ldk, long long kofs, int tf32,
-                        cudaStream_t st, int variant = 0, unsigned* absmax = nullptr);
+void launch_mgen(const LriGeom& g, const cplx<T>* T1, const cplx<T>* evec, int q, int kk0, int nkk, MapMode mode, int a0,
+                 int na, int b0, int nb, cplx<T>* out, long long s_r, long long s_mu, cudaStream_t st,
+                 unsigned* absmax = nullptr);
 
 // k_linalg.cu
 template <typename T>
@@ -108,7 +93,7 @@ gw_status launch_inv_minus_I(int N, c128* A, int batch, long long stride, void* 
 template <typename T> void launch_axpby_identity(int N, cplx<T>* A, long long s, int batch, T diag, cudaStream_t st);
 void launch_take_both(int N, const c128* C, long long s, int batch, float d, c64* X, c64* XH, cudaStream_t st);
 void launch_dev_identity(int N, const c64* T, long long total, unsigned* dev, cudaStream_t st);
-void launch_convert(int n, const c128* in, c64* out, cudaStream_t st);
+void launch_convert(long long n, const c128* in, c64* out, cudaStream_t st);
 // dominant eigenpair of a Hermitian matrix by power iteration (FP64)
 void launch_power_iter(int N, const c128* A, c128* x, double* lam, int iters, cudaStream_t st);
 // A += alpha * x x^H

@@ -1,6 +1,6 @@
 // CUDA-core linear algebra of the G0W0 path: the generic complex GEMM used by the
 // FP64 method and by the V^1/2 Newton-Schulz iteration, the FP64 chi0 contraction,
-// the FP64 Cholesky factorisation + inversion of eps~, and the q = 0 helpers.
+// and the q = 0 helpers.
 #include "gw_internal.h"
 
 namespace gw {
@@ -351,12 +351,12 @@ void launch_take_both(int N, const c128* C, long long s, int batch, float d, c64
   ++::gw::g_launch_count, k_take_both<<<grid, dim3(32, 8), 0, st>>>(N, C, s, d, X, XH);
 }
 
-__global__ void k_convert(int n, const c128* in, c64* out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+__global__ void k_convert(long long n, const c128* in, c64* out) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = c64{(float)in[i].re, (float)in[i].im};
 }
-void launch_convert(int n, const c128* in, c64* out, cudaStream_t st) {
-  ++::gw::g_launch_count, k_convert<<<std::min((n + 255) / 256, 152 * 32), 256, 0, st>>>(n, in, out);
+void launch_convert(long long n, const c128* in, c64* out, cudaStream_t st) {
+  ++::gw::g_launch_count, k_convert<<<(int)std::min<long long>((n + 255) / 256, 152LL * 32), 256, 0, st>>>(n, in, out);
 }
 
 // Dominant eigenpair by power iteration with a Rayleigh quotient (one block, FP64). Each warp
