@@ -25,9 +25,11 @@
 // faster than one FP64 one. What is left in FP64 is one addition per element and pivot block, and
 // the factor of the 32 x 32 pivot blocks. Every size is spread over the whole chip (a CTA per 64 rows
 // of a matrix). Measured against one block per matrix with FP64 FMAs throughout: 1152 matrices of
-// N = 400 332 -> 63 ms, 32 of them 44 -> 2.6 ms, 16 of N = 1200 1004 -> 14 ms, 32 of N = 96 1.5 -> 0.4 ms;
+// N = 400 332 -> 47 ms, 32 of them 44 -> 2.1 ms, 16 of N = 1200 1004 -> 10.6 ms, 32 of N = 96 1.5 -> 0.4 ms;
 // the error against a refined inverse is the same (N = 400: 3.7e-16 and 5.6e-16 before at kappa = 3,
-// 4.7e-10 and 6.5e-10 before at kappa = 2e7).
+// 4.7e-10 and 6.5e-10 before at kappa = 2e7). Two thirds of it are the updates, which take ~9 us per 64 x 64
+// tile: the products need 2, the FP64 conversions and additions of the epilogue 3, the rest is latency
+// (loads of B, the handover of the accumulators, the left operand at the start of a row block).
 #include "gw_internal.h"
 #include "tc_ptx.cuh"
 
@@ -113,19 +115,9 @@ __device__ __forceinline__ uint4 neg8(uint4 v) {
   return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
 }
 
-// T 2^ex rounded to FP64 (integer arithmetic only)
-__device__ __forceinline__ double pack_double(long long T, int ex) {
-  if (ex > E_BAD / 2) return __longlong_as_double(0x7ff8000000000000LL);
-  if (T == 0) return 0.0;
-  unsigned long long u = T < 0 ? (unsigned long long)(-T) : (unsigned long long)T;
-  const int lz = __clzll((long long)u);
-  u <<= lz;
-  const unsigned long long m = (u >> 11) + ((u >> 10) & 1);
-  const int f = ex + 63 - lz + 1022;
-  if (f < 0) return 0.0;
-  if (f >= 2046) return __longlong_as_double(0x7ff8000000000000LL);
-  const unsigned long long bits = ((unsigned long long)f << 52) + m;
-  return __longlong_as_double((long long)(bits | (T < 0 ? 0x8000000000000000ULL : 0ULL)));
+// 2^ex, 0 below the normal range and infinity above it
+__device__ __forceinline__ double pow2(int ex) {
+  return __hiloint2double(max(0, min(ex + 1023, 2047)) << 20, 0);
 }
 
 __host__ __device__ __forceinline__ int padded(int N) { return (N + TM - 1) / TM * TM; }
@@ -270,71 +262,79 @@ struct InvMaps {
   CUtensorMap yb, ya, w, r;
 };
 
-__device__ __forceinline__ void ld16(uint32_t taddr, int (&v)[16]) {
-  uint32_t r[16];
+// 256 v_o + v_(o+1) of 16 columns. SMALL: |v| <= 2^22 (orders 0-3: at most 4 pairs x 2^20), converted by
+// an exact addition of 1.5 2^23 whose bits hold the integer (the general conversion runs at a quarter rate)
+template <bool SMALL, int STRIDE> __device__ __forceinline__ void ld_pair(uint32_t taddr, int (&v)[16]) {
+  uint32_t r[16], s[16];
   tmem_ld16_nowait(taddr, r);
+  tmem_ld16_nowait(taddr + STRIDE, s);
   tmem_wait_ld();
 #pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = __float2int_rn(__uint_as_float(r[j]));
+  for (int j = 0; j < 16; ++j) {
+    const float x = __uint_as_float(r[j]), y = __uint_as_float(s[j]);
+    if constexpr (SMALL)
+      v[j] = __float_as_int(x + 12582912.0f) * 256 + __float_as_int(y + 12582912.0f) - 0x4b400000 * 257u;
+    else
+      v[j] = __float2int_rn(x) * 256 + __float2int_rn(y);
+  }
 }
-// orders 0-3 of 16 columns: S = sum_o v_o 256^(3 - o)  (|S| < 2^45)
-__device__ __forceinline__ void high_orders(uint32_t tl, long long (&S)[16]) {
+// orders 0-3 of 16 columns (orders STRIDE columns apart): S = sum_o v_o 256^(3 - o)  (|S| < 2^45)
+template <int STRIDE> __device__ __forceinline__ void high_orders(uint32_t tl, long long (&S)[16]) {
   int v[16], w[16];
-  ld16(tl, v);
-  ld16(tl + TM, w);
+  ld_pair<true, STRIDE>(tl, v);
+  ld_pair<true, STRIDE>(tl + 2 * STRIDE, w);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) S[j] = (long long)(v[j] * 256 + w[j]) * 65536;
-  ld16(tl + 2 * TM, v);
-  ld16(tl + 3 * TM, w);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) S[j] += v[j] * 256 + w[j];
+  for (int j = 0; j < 16; ++j) S[j] = (long long)v[j] * 65536 + w[j];
 }
 // and orders 4-6: S <- (S 2^24 + sum_o v_o 256^(6 - o)) / 64  (|S| < 2^63)
-__device__ __forceinline__ void low_orders(uint32_t tl, long long (&S)[16]) {
-  int v[16], w[16];
-  ld16(tl + 4 * TM, v);
-  ld16(tl + 5 * TM, w);
+template <int STRIDE> __device__ __forceinline__ void low_orders(uint32_t tl, long long (&S)[16]) {
+  int v[16];
+  uint32_t r[16];
+  tmem_ld16_nowait(tl + 6 * STRIDE, r);
+  ld_pair<false, STRIDE>(tl + 4 * STRIDE, v);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = v[j] * 256 + w[j];
-  ld16(tl + 6 * TM, w);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) S[j] = (S[j] << 18) + (((long long)v[j] * 256 + w[j]) >> 6);
+  for (int j = 0; j < 16; ++j)
+    S[j] = (S[j] << 18) + (((long long)v[j] * 256 + __float2int_rn(__uint_as_float(r[j]))) >> 6);
 }
 // A lane of the upper half holds Im, of the lower half Re of the same row: for the column pair
 // (2u, 2u + 1) the lower half keeps column 2u and the upper half 2u + 1, each with both parts
-__device__ __forceinline__ double2 trade(const long long s0, const long long s1, int h, int ex) {
+// (integers below 2^63, rounded to FP64 once)
+__device__ __forceinline__ double2 trade(const long long s0, const long long s1, int h) {
   const long long got = __shfl_xor_sync(0xffffffffu, h ? s0 : s1, 16);
-  return make_double2(pack_double(h ? got : s0, ex), pack_double(h ? s1 : got, ex));
+  return make_double2((double)(h ? got : s0), (double)(h ? s1 : got));
 }
 constexpr int E_SHIFT = 110 - 48 - 6;    // value = S 2^(e_left + e_right - E_SHIFT)
 
-// ---- Y_i = B_iP W^H and its digits, 64 rows per CTA ---------------------------------------------
+// ---- Y_i = B_iP W^H and its digits, 32 rows per CTA ---------------------------------------------
 //
 // The panel rows are read and cut straight into the right operand in shared memory, W is the left
-// one (conj(Y_i) = W B_iP^H, so only W needs stacked rows), and the product's rows are cut again.
-constexpr int Y_THREADS = 512;
+// one (conj(Y_i) = W B_iP^H, so only W needs stacked rows), and the product's rows are cut again. The
+// steps of a CTA follow one another, so two CTAs share an SM (110 KB and 256 TMEM columns each).
+constexpr int YR = 32;                                       // rows per CTA
+constexpr int Y_THREADS = 8 * YR;
+constexpr int Y_PIECE = YR * ROWB;
 constexpr int Y_OFF_B = ND * W_PLANE + W_PLANE;              // (the MMA reads 128 rows of a 64-row digit)
-constexpr int Y_OFF_Z = Y_OFF_B + ND * B_PIECE;
-constexpr int Y_OFF_E = Y_OFF_Z + PB * (TM + 1) * 16;
-constexpr int Y_OFF_BAR = Y_OFF_E + TM * 4;
+constexpr int Y_OFF_Z = Y_OFF_B + ND * Y_PIECE;
+constexpr int Y_OFF_E = Y_OFF_Z + PB * (YR + 1) * 16;
+constexpr int Y_OFF_BAR = Y_OFF_E + YR * 4;
 constexpr int Y_SMEM = Y_OFF_BAR + 32 + 1024;
-static_assert(Y_SMEM <= 232448, "shared memory budget");
+static_assert(2 * (Y_SMEM + 1024) <= 233472, "two blocks per SM");
 
-__global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ InvMaps maps, int N, int Nr, int p, int batch,
+__global__ void __launch_bounds__(Y_THREADS, 2) k_inv_y(const __grid_constant__ InvMaps maps, int N, int Nr, int p, int batch,
                                                         const c128* __restrict__ Aall, long long stride,
                                                         uint8_t* __restrict__ yb, uint8_t* __restrict__ ya,
                                                         const int* __restrict__ eW, int* __restrict__ eY,
                                                         int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  double2* Z = reinterpret_cast<double2*>(smem + Y_OFF_Z);     // [32 panel columns][65 rows], then [64][32]
+  double2* Z = reinterpret_cast<double2*>(smem + Y_OFF_Z);     // [32 panel columns][33 rows], then [32][32]
   int* eC = reinterpret_cast<int*>(smem + Y_OFF_E);
   uint64_t* wfull = reinterpret_cast<uint64_t*>(smem + Y_OFF_BAR);
   uint64_t* dfull = wfull + 1;
   uint32_t* tmem_p = reinterpret_cast<uint32_t*>(wfull + 2);
   const int t = threadIdx.x, warp = t / 32, lane = t % 32;
   const int blk = blockIdx.x / batch, b = blockIdx.x % batch;
-  const int r0 = blk * TM, pw = min(PB, N - p);
+  const int r0 = blk * YR, pw = min(PB, N - p);
   const c128* A = Aall + b * stride;
   if (t == 0) {
     mbar_init(wfull, 1);
@@ -344,12 +344,12 @@ __global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ 
     for (int d = 0; d < ND; ++d) tma_load_2d(smem + d * W_PLANE, &maps.w, wfull, 0, (b * ND + d) * 2 * PB);
   }
   if (warp == 1) {
-    tmem_alloc(tmem_p, 512);
+    tmem_alloc(tmem_p, 256);
     tmem_relinquish();
   }
-  for (int e = t; e < TM * PB; e += Y_THREADS) {
+  for (int e = t; e < YR * PB; e += Y_THREADS) {
     // behind the pivot the panel runs along the rows, before it along the panel columns
-    int r = e % TM, c = e / TM;
+    int r = e % YR, c = e / YR;
     if (r0 < p) {
       r = e / PB;
       c = e % PB;
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ 
         z = make_double2(a.re, -a.im);
       }
     }
-    Z[c * (TM + 1) + r] = z;
+    Z[c * (YR + 1) + r] = z;
   }
   __syncthreads();
   const int r = t >> 3, part = (t >> 2) & 1, qr = t & 3;      // 8 threads per row: Re / Im, a quarter of the columns
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ 
     double x[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      const double2 z = Z[(8 * qr + c) * (TM + 1) + r];
+      const double2 z = Z[(8 * qr + c) * (YR + 1) + r];
       x[c] = part ? z.y : z.x;
     }
     int e;
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ 
 #pragma unroll
     for (int c = 0; c < 8; ++c) y[c] = to_digits(x[c], f);
     each_digit<0>(y, [&](int d, uint4 q) {
-      *reinterpret_cast<uint4*>(smem + Y_OFF_B + d * B_PIECE + swz(r, part * 4 + qr)) = q;
+      *reinterpret_cast<uint4*>(smem + Y_OFF_B + d * Y_PIECE + swz(r, part * 4 + qr)) = q;
     });
     fence_proxy_async();
   }
@@ -392,16 +392,16 @@ __global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ 
   tc_fence_after();
   const uint32_t tmem = *tmem_p;
   if (t == 0) {
-    const uint32_t idesc = (1u << 4) | ((uint32_t)(TM >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    const uint32_t idesc = (1u << 4) | ((uint32_t)(YR >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     const uint32_t abase = smem_u32(smem), bbase = abase + Y_OFF_B;
     if (mbar_wait(wfull, 0, status)) {
       tc_fence_after();
       for (int o = 0; o < ND; ++o)
         for (int d1 = 0; d1 <= o; ++d1) {
-          const uint64_t dA = sdesc(abase + d1 * W_PLANE), dB = sdesc(bbase + (o - d1) * B_PIECE);
+          const uint64_t dA = sdesc(abase + d1 * W_PLANE), dB = sdesc(bbase + (o - d1) * Y_PIECE);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            mma<false>(tmem + o * TM, dA + 2 * kk, dB + 2 * kk, idesc, (d1 == 0 && kk == 0) ? 0u : 1u);
+            mma<false>(tmem + o * YR, dA + 2 * kk, dB + 2 * kk, idesc, (d1 == 0 && kk == 0) ? 0u : 1u);
         }
     }
     mma_commit(dfull);
@@ -414,20 +414,21 @@ __global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ 
     const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + cg * 16;
     const int pc = quad * 16 + (lane & 15);
     long long S[16];
-    high_orders(tl, S);
-    low_orders(tl, S);
+    high_orders<YR>(tl, S);
+    low_orders<YR>(tl, S);
     const int ew = eW[b * PB + pc] - E_SHIFT;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int c = cg * 16 + 2 * u + h;                       // row of the block
-      const double2 z = trade(S[2 * u], S[2 * u + 1], h, ew + eC[c]);
-      Z[c * PB + pc] = make_double2(z.x, -z.y);
+      const double2 z = trade(S[2 * u], S[2 * u + 1], h);
+      const double f = pow2(ew + eC[c]);
+      Z[c * PB + pc] = make_double2(f * z.x, -f * z.y);
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, 512);
+  if (warp == 1) tmem_dealloc(tmem, 256);
   double x[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
@@ -440,10 +441,10 @@ __global__ void __launch_bounds__(Y_THREADS, 1) k_inv_y(const __grid_constant__ 
   long long y[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) y[c] = to_digits(x[c], f);
-  const int m1 = (r >> 4) * 32 + (r & 15), m2 = m1 + 16;
+  const int r64 = r0 % TM + r, m1 = (r64 >> 4) * 32 + (r64 & 15), m2 = m1 + 16;
   const int nblk = Nr / TM;
   uint8_t* ob = yb + ((long long)b * ND * Nr + r0 + r) * ROWB + (part * 4 + qr) * 16;
-  uint8_t* oa = ya + ((long long)b * ND * nblk + blk) * A_PIECE;
+  uint8_t* oa = ya + ((long long)b * ND * nblk + r0 / TM) * A_PIECE;
   each_digit<0>(y, [&](int d, uint4 q) {
     *reinterpret_cast<uint4*>(ob + (long long)d * Nr * ROWB) = q;
     uint8_t* o = oa + (long long)d * nblk * A_PIECE;
@@ -556,46 +557,57 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_inv_update(const __grid_cons
     const int pw = min(PB, N - p);
     const bool rok = row < N && !(row >= p && row < p + PB);
     const int erow = eY[(long long)b * Nr + row] - E_SHIFT;
+    const bool full_rows = bi * TM + quad * 16 + 16 <= p || bi * TM + quad * 16 >= p + PB;   // none of the warp's in P
     for (int tt = 0; tt < ntile; ++tt) {
       const bool panel = tt == 0;
       const bool active = !panel || cg < 2;           // the panel has 32 columns
       // the elements this thread updates: columns c0 + 2 u + h, u < 8
       const int c0 = panel ? cg * 16 : (tt - 1) * TM + cg * 16;
-      c128 old[8];
-      int ecol[8];
+      c128* at = A + (long long)(c0 + h) * N + row;                // and every second column of B from there
+      const int* et = panel ? eR + b * PB : eY + (long long)b * Nr;
+      // whole tiles left of the diagonal and off the pivot block take every element
       unsigned live = 0;
+      if (!panel && bi * TM + TM <= N && c0 + 16 <= bi * TM && (c0 >= p + PB || c0 + 16 <= p) && full_rows) {
+        live = 0xffu;
+      } else if (rok) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int c = c0 + 2 * u + h;
-        const bool lv = rok && (panel ? c < pw : c <= row && !(c >= p && c < p + PB));
-        if (lv) {
-          live |= 1u << u;
-          if (!panel) old[u] = A[(long long)c * N + row];
+        for (int u = 0; u < 8; ++u) {
+          const int c = c0 + 2 * u + h;
+          live |= (panel ? c < pw : c <= row && !(c >= p && c < p + PB)) ? 1u << u : 0u;
         }
-        ecol[u] = panel ? (active ? eR[b * PB + c] : 0) : eY[(long long)b * Nr + c];
       }
+      c128 old[4];
       long long S[16];
       if (!__all_sync(0xffffffffu, mbar_wait(&dfull[0], tt & 1, status))) break;
       tc_fence_after();
-      if (active) high_orders(tl, S);
+      if (active) high_orders<TM>(tl, S);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&dempty[0]);
+      if (!panel)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (live & (1u << u)) old[u] = at[2LL * u * N];
       if (!__all_sync(0xffffffffu, mbar_wait(&dfull[1], tt & 1, status))) break;
       tc_fence_after();
-      if (active) low_orders(tl, S);
+      if (active) low_orders<TM>(tl, S);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&dempty[1]);
       if (active) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const double2 z = trade(S[2 * u], S[2 * u + 1], h, erow + ecol[u]);
-          if (live & (1u << u)) {
-            const int c = c0 + 2 * u + h;
-            if (!panel) A[(long long)c * N + row] = c128{old[u].re - z.x, old[u].im - z.y};
-            else if (row >= p) A[(long long)(p + c) * N + row] = c128{z.x, z.y};
-            else A[(long long)row * N + p + c] = c128{z.x, -z.y};
+        for (int g = 0; g < 2; ++g) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int u = 4 * g + v, c = c0 + 2 * u + h;
+            const double2 z = trade(S[2 * u], S[2 * u + 1], h);
+            const double f = pow2(erow + et[c]);
+            if (live & (1u << u)) {
+              if (!panel) at[2LL * u * N] = c128{fma(-f, z.x, old[v].re), fma(-f, z.y, old[v].im)};
+              else if (row >= p) A[(long long)(p + c) * N + row] = c128{f * z.x, f * z.y};
+              else A[(long long)row * N + p + c] = c128{f * z.x, -f * z.y};
+            }
+            if (g == 0 && !panel && (live & (16u << v))) old[v] = at[2LL * (u + 4) * N];
           }
         }
       }
@@ -655,7 +667,7 @@ gw_status launch_inv_minus_I(int N, c128* A, int batch, long long stride, void* 
   for (int p = 0; p < N; p += PB) {
     ++g_launch_count, k_inv_pivot<<<batch, PIV_THREADS, 0, st>>>(N, p, A, stride, w + l.w, w + l.r, eW, eR, status);
     if (N <= PB) break;
-    ++g_launch_count, k_inv_y<<<nblk * batch, Y_THREADS, Y_SMEM, st>>>(maps, N, Nr, p, batch, A, stride, w + l.yb,
+    ++g_launch_count, k_inv_y<<<Nr / YR * batch, Y_THREADS, Y_SMEM, st>>>(maps, N, Nr, p, batch, A, stride, w + l.yb,
                                                                       w + l.ya, eW, eY, status);
     ++g_launch_count, k_inv_update<<<nblk * batch, UPD_THREADS, UPD_SMEM, st>>>(maps, N, Nr, p, batch, A, stride, eY, eR,
                                                                                status);
