@@ -65,14 +65,15 @@ __global__ void k_sigma_conv(int kk0, int nsig, int NBd, int n1, int n2, int n3,
     for (int m = part; m < NBd; m += parts) {
       const long long r = ((long long)kk * nsig + n) * NBd + m;
       const T zr = mu - (T)eps[(long long)kmq * NBd + m];   // z = zr + i om
-      // z^2 + w_j^2 = zr^2 + (w_j - om)(w_j + om) + 2 i zr om (no cancellation of the two squares)
-      const T zr2 = zr * zr, di = (T)2 * zr * om;
+      // z^2 = zr^2 - om^2 + 2 i zr om
+      const T z2r = zr * zr - om * om, z2i = (T)2 * zr * om;
       T sr = 0, si = 0;
 #pragma unroll 4
       for (int j = 0; j < nw; ++j) {
         const T s = gg[j] * (S_d ? (T)S_d[r * nw + j] : (T)S_f[r * nw + j]);
         // 2 z / (z^2 + wj^2)
-        const T dr = zr2 + (fr[j] - om) * (fr[j] + om);
+        const T wj = fr[j];
+        const T dr = z2r + wj * wj, di = z2i;
         const T inv = (T)1 / (dr * dr + di * di);
         const T fr_ = (T)2 * (zr * dr + om * di) * inv;
         const T fi_ = (T)2 * (om * dr - zr * di) * inv;
