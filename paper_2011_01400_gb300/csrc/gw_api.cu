@@ -262,9 +262,10 @@ struct gw_plan_s {
   int* d_eB = nullptr;        // FP16: exponent of the B plane scale
   double* d_escale = nullptr; // [nw] factors of the drained chi0 sums
   Chi0Plan* chi0plan = nullptr;   // work lists of the tcgen05 chi0 kernel (and the screen products)
-  float* d_hb[2] = {nullptr, nullptr};  // screen products: TF32 pieces of the Hermitian right operand
-  float* d_hones = nullptr;             // [Kpad] unit weights
-  double* d_hesc = nullptr;             // [nw]
+  // screen products: the left operands' largest elements [2][nw], weight rows [nw][Kpad] and factors [nw]
+  unsigned* d_hmax = nullptr;
+  float* d_hrow = nullptr;
+  double* d_hesc = nullptr;
   // frequency compression of the split-precision chi0 (k_compress.cu)
   // largest relative residual |W_j - sum_{t<T} E_jt v_t| / |W_j| over the frequencies j that the
   // compression may leave (computed in FP64 over all pair rows); 0 disables. 3e-8 is below the
@@ -280,8 +281,10 @@ struct gw_plan_s {
   int last_T = 0;             // components kept for the last q
   int Kx = 0;                 // n_aux rounded up to 32 (K of the Sigma contraction)
   PlaneSet d_Wpl{};           // W^c split planes [nw*N][2*Kx]
-  c64* d_Vh32 = nullptr;      // FP32 copies of V^1/2 for the split-precision screen
-  c64* d_Vb32 = nullptr;
+  // FP16 pieces of V(q)^1/2 [NK N][2 Kpad] (and of d_Vb0, one matrix more at the end) and their scales, the
+  // right operand of every screen product
+  uint16_t* d_Vpc[2] = {nullptr, nullptr};
+  int* d_Ve = nullptr;
   // q-group buffers of gw_g0w0
   c128 *g_chi0 = nullptr, *g_E = nullptr;
   uint8_t* g_work = nullptr;
@@ -435,21 +438,33 @@ gw_status newton_schulz(gw_plan_s* P, const c128* V, c128* out, int batch, int i
   return GW_OK;
 }
 
-gw_status herm_gemm(gw_plan_s* P, const c64* A, bool a_batch, const c128* H64, const c64* H32, bool h_batch,
-                    double alpha, c128* C, int nb);
+// one product of the kernel with a status and an error text
+gw_status herm_gemm(gw_plan_s* P, const HermGemmArgs& g) {
+  std::string err;
+  gw_status ts = herm_gemm_run(g, &P->chi0plan, P->st, err);
+  if (ts != GW_OK) {
+    P->err = 1;
+    return fail(ts, "screen product: " + err);
+  }
+  return GW_OK;
+}
 
 // The same iteration on the tensor cores for the split path: its three products per step as TF32
-// two-piece products, FP64-accumulated, in chunks of n_freq matrices (the screen's product
-// workspace). The kernel multiplies by the conjugate transpose of the rows it is given, so every
-// right operand goes in as its conjugate transpose, written next to it when it is formed. (Y, Z and
-// T are Hermitian in exact arithmetic, but taking H^H for H, or projecting them on their Hermitian
-// parts, turns the rounding into a mode that grows after convergence; the plain products do not.)
+// two-piece products, FP64 out, in chunks of n_freq matrices. The kernel
+// multiplies by the conjugate transpose of the rows it is given and writes the conjugate transpose of
+// the product, so every operand is kept with its conjugate transpose next to it. (Y, Z and T are
+// Hermitian in exact arithmetic, but taking H^H for H, or projecting them on their Hermitian parts, turns
+// the rounding into a mode that grows after convergence; the plain products do not.)
 gw_status newton_schulz_tc(gw_plan_s* P, c128* Vio, int batch, int iters) {
   const int N = P->N, nb = P->nw;
   const long long s = (long long)N * N;
+  const size_t Kpad = (size_t)(N + 31) / 32 * 32;
   double* d_c;
   c64 *Y, *Yh, *Z, *Zh, *Tm, *Th;
   c128* C;
+  float* pc[2];
+  unsigned* d_dev;
+  const size_t held = P->allocs.size();
   GW_TRY(dalloc(P, &d_c, batch));
   GW_TRY(dalloc(P, &Y, s * nb));
   GW_TRY(dalloc(P, &Yh, s * nb));
@@ -458,8 +473,27 @@ gw_status newton_schulz_tc(gw_plan_s* P, c128* Vio, int batch, int iters) {
   GW_TRY(dalloc(P, &Tm, s * nb));
   GW_TRY(dalloc(P, &Th, s * nb));
   GW_TRY(dalloc(P, &C, s * nb));
-  unsigned* d_dev;
+  for (auto& p : pc) GW_TRY(dalloc(P, &p, (size_t)nb * N * 2 * Kpad));
   GW_TRY(dalloc(P, &d_dev, 1));
+  // X, X^H <- alpha A H + d 1, H given by its conjugate transpose Hh
+  auto product = [&](const c64* A, const c64* Hh, double alpha, float d, c64* X, c64* XH, int n) -> gw_status {
+    herm_pieces_tf32(N, n, Hh, pc[0], pc[1], P->st);
+    HermGemmArgs g{};
+    g.N = N;
+    g.nb = n;
+    g.A = A;
+    g.h[0] = pc[0];
+    g.h[1] = pc[1];
+    g.h_batch = 1;
+    g.alpha = alpha;
+    g.C = C;
+    g.wrow = P->d_hrow;
+    g.escale = P->d_hesc;
+    g.status = P->d_status;
+    GW_TRY(herm_gemm(P, g));
+    launch_take_both(N, C, s, n, d, XH, X, P->st);   // C holds the conjugate transpose
+    return GW_OK;
+  };
   ++::gw::g_launch_count, k_frob_scale<<<batch, 256, 0, P->st>>>(N, Vio, s, d_c);
   for (int b0 = 0; b0 < batch; b0 += nb) {
     const int n = std::min(nb, batch - b0);
@@ -471,8 +505,7 @@ gw_status newton_schulz_tc(gw_plan_s* P, c128* Vio, int batch, int iters) {
       return fail(GW_ERR_CUDA, "newton_schulz: copy failed");
     for (int it = 0; it < iters; ++it) {
       // T = 1.5 I - 0.5 Z Y;  Y <- Y T;  Z <- T Z
-      GW_TRY(herm_gemm(P, Z, true, nullptr, Yh, true, -0.5, C, n));
-      launch_take_both(N, C, s, n, 1.5f, Tm, Th, P->st);
+      GW_TRY(product(Z, Yh, -0.5, 1.5f, Tm, Th, n));
       // converged chunk: once max |T - I| < 1e-4 the step below leaves it ~1e-8 from I (the
       // iteration converges quadratically), below the FP32 rounding of the products
       bool last = false;
@@ -487,18 +520,16 @@ gw_status newton_schulz_tc(gw_plan_s* P, c128* Vio, int batch, int iters) {
         std::memcpy(&dev, &hdev, sizeof(float));
         last = dev < 1e-4f;
       }
-      GW_TRY(herm_gemm(P, Y, true, nullptr, Th, true, 1.0, C, n));
-      launch_take_both(N, C, s, n, 0.0f, Y, Yh, P->st);
+      GW_TRY(product(Y, Th, 1.0, 0.0f, Y, Yh, n));
       if (last) break;
-      GW_TRY(herm_gemm(P, Tm, true, nullptr, Zh, true, 1.0, C, n));
-      launch_take_both(N, C, s, n, 0.0f, Z, Zh, P->st);
+      GW_TRY(product(Tm, Zh, 1.0, 0.0f, Z, Zh, n));
     }
     ++::gw::g_launch_count, k_ns_final<float><<<g, 256, 0, P->st>>>(N, Y, s, d_c + b0, Vio + b0 * s);
   }
   GW_TRY(check_launch(P, "newton_schulz"));
   cudaError_t e = cudaStreamSynchronize(P->st);
   if (e != cudaSuccess) return fail(GW_ERR_CUDA, std::string("newton_schulz: ") + cudaGetErrorString(e));
-  for (int i = 0; i < 9; ++i) dfree_last(P);
+  while (P->allocs.size() > held) dfree_last(P);
   return GW_OK;
 }
 
@@ -803,26 +834,18 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
       ALLOC(pp, we);
       P->d_Wpl.b[i] = pp;
     }
-    c64 *v32, *b32;
-    ALLOC(v32, NN * P->NK);
-    P->d_Vh32 = v32;
-    if (prob->head_wings) {
-      ALLOC(b32, NN);
-      P->d_Vb32 = b32;
-    }
+    const size_t vp = (size_t)(P->NK + (prob->head_wings ? 1 : 0)) * N;
+    for (auto& p : P->d_Vpc) ALLOC(p, vp * 2 * P->Kx);
+    ALLOC(P->d_Ve, vp / N);
   }
   if (!P->fp64) {
     const size_t pe = (size_t)N * 2 * P->ldm * (P->prec == GW_3XTF32 ? 4 : 2);
     ALLOC(P->d_Praw, (size_t)N * 2 * P->ldm);
     P->n_bpl = P->prec == GW_3XBF16 ? 3 : 2;
     ALLOC(P->d_absmax, 1);
-    {
-      const size_t kp = (size_t)(N + 31) / 32 * 32;
-      ALLOC(P->d_hb[0], (size_t)nw * N * 2 * kp);
-      ALLOC(P->d_hb[1], (size_t)nw * N * 2 * kp);
-      ALLOC(P->d_hones, kp);
-      ALLOC(P->d_hesc, (size_t)nw);
-    }
+    ALLOC(P->d_hmax, std::max<size_t>(2 * (size_t)nw, P->NK + 1));
+    ALLOC(P->d_hrow, (size_t)nw * P->Kx);
+    ALLOC(P->d_hesc, (size_t)nw);
     ALLOC(P->d_eB, 1);
     ALLOC(P->d_escale, (size_t)nw);
     for (int i = 0; i < P->n_bpl; ++i) {
@@ -963,8 +986,15 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
   }
   if (!P->fp64) {
     launch_convert((long long)P->NK * P->NB * P->NBd, reinterpret_cast<const c128*>(prob->evec), P->d_evec32, st);
-    launch_convert((long long)NN * P->NK, P->d_Vh, P->d_Vh32, st);
-    if (prob->head_wings) launch_convert((long long)NN, P->d_Vb0, P->d_Vb32, st);
+    // pieces of V^1/2 (d_hmax holds the largest elements meanwhile)
+    auto pieces = [&](const c128* V, int mats, size_t m0) {
+      const size_t o = m0 * N * 2 * P->Kx;
+      herm_round_max((long long)NN, mats, V, nullptr, P->d_hmax + m0, st);
+      herm_pieces_f16(N, mats, V, P->d_hmax + m0, P->d_Vpc[0] + o, P->d_Vpc[1] + o, P->d_Ve + m0, st);
+    };
+    CK(cudaMemsetAsync(P->d_hmax, 0, sizeof(unsigned) * (P->NK + 1), st));
+    for (int q0 = 0; q0 < P->NK; q0 += 32768) pieces(P->d_Vh + q0 * NN, std::min(32768, P->NK - q0), q0);
+    if (prob->head_wings) pieces(P->d_Vb0, 1, P->NK);
     CK(cudaMemsetAsync(P->d_A, 0, sizeof(c64) * (size_t)P->sig_rows * P->Kx, st));
   }
   if ((s = check_launch(P, "plan setup")) != GW_OK) return cleanup(s);
@@ -1223,35 +1253,39 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
   return GW_OK;
 }
 
-// C[b] = alpha A[b] H[b] for b < nb on the tensor cores (split precision screen products; H
-// Hermitian, FP64 or FP32)
-gw_status herm_gemm(gw_plan_s* P, const c64* A, bool a_batch, const c128* H64, const c64* H32, bool h_batch,
-                    double alpha, c128* C, int nb) {
+// out[b] = alpha S X[b] S + diag 1 for the nw matrices X[b] (FP64, Hermitian) and S = matrix m of the plan's
+// V^1/2 pieces (Hermitian): two tensor-core products. The first, X S, leaves its conjugate transpose S X in
+// FP32, the left operand of the second; the second leaves (S X S)^H.
+gw_status sandwich(gw_plan_s* P, const c128* X, size_t m, double alpha, double diag, c128* out) {
+  cudaStream_t st = P->st;
+  const int N = P->N, nw = P->nw;
+  const long long NN = (long long)N * N;
+  c64* A32 = reinterpret_cast<c64*>(P->d_work);
+  c64* B32 = A32 + NN * nw;
+  GW_CUDA(cudaMemsetAsync(P->d_hmax, 0, 2 * sizeof(unsigned) * nw, st));
+  herm_round_max(NN, nw, X, A32, P->d_hmax, st);
   HermGemmArgs g{};
-  g.N = P->N;
-  g.nb = nb;
-  g.A = A;
-  g.a_batch = a_batch ? 1 : 0;
-  g.H64 = H64;
-  g.H32 = H32;
-  g.h_batch = h_batch ? 1 : 0;
-  g.alpha = alpha;
-  g.C = C;
-  g.bpl[0] = P->d_hb[0];
-  g.bpl[1] = P->d_hb[1];
-  g.ones = P->d_hones;
+  g.N = N;
+  g.nb = nw;
+  g.A = A32;
+  g.f16 = 1;
+  g.amaxA = P->d_hmax;
+  for (int i = 0; i < 2; ++i) g.h[i] = P->d_Vpc[i] + m * N * 2 * P->Kx;
+  g.eB = P->d_Ve + m;
+  g.alpha = 1.0;
+  g.C32 = B32;
+  g.amaxC = P->d_hmax + nw;
+  g.wrow = P->d_hrow;
   g.escale = P->d_hesc;
   g.status = P->d_status;
-  std::string err;
-  gw_status ts = herm_gemm_run(g, &P->chi0plan, P->st, err);
-  if (ts != GW_OK) {
-    P->err = 1;
-    return fail(ts, "screen product: " + err);
-  }
-  return GW_OK;
-}
-gw_status herm_gemm(gw_plan_s* P, const c64* A, bool a_batch, const c128* H, bool h_batch, double alpha, c128* C) {
-  return herm_gemm(P, A, a_batch, H, nullptr, h_batch, alpha, C, P->nw);
+  GW_TRY(herm_gemm(P, g));
+  g.A = B32;
+  g.amaxA = P->d_hmax + nw;
+  g.alpha = alpha;
+  g.diag = diag;
+  g.C32 = nullptr;
+  g.C = out;
+  return herm_gemm(P, g);
 }
 
 // E[b] := E[b]^{-1} - 1 for `batch` matrices eps~ (FP64)
@@ -1274,20 +1308,13 @@ gw_status eps_core(gw_plan_s* P, int q, const c128* chi0, c128* E) {
   const c128* Vh = P->d_Vh + (long long)q * NN;
   const c128* Vin = hw ? P->d_Vb0 : Vh;     // V^1/2 entering eps~ (body only at q = 0)
   const c128 one{1, 0}, zero{0, 0}, mone{-1, 0};
-  c64* A32 = reinterpret_cast<c64*>(P->d_work);
   if (P->fp64) {
     launch_zgemm<double>(N, N, N, one, chi0, N, NN, OP_N, Vin, N, 0, OP_N, zero, P->d_tmp, N, NN, nw, st);
     launch_zgemm<double>(N, N, N, mone, Vin, N, 0, OP_N, P->d_tmp, N, NN, OP_N, zero, E, N, NN, nw, st);
   } else {
-    // V^1/2 chi0 V^1/2 as (V^1/2 chi0) V^1/2: both right operands are Hermitian, the form of the
-    // tensor-core kernel (TF32 two-piece products, FP64 accumulation)
-    const c64* Vh32 = P->d_Vh32 + (long long)q * NN;
-    const c64* Vin32 = hw ? P->d_Vb32 : Vh32;
-    GW_TRY(herm_gemm(P, Vin32, false, chi0, true, 1.0, P->d_tmp));
-    launch_convert(NN * nw, P->d_tmp, A32, st);
-    GW_TRY(herm_gemm(P, A32, true, Vin, false, -1.0, E));
+    GW_TRY(sandwich(P, chi0, hw ? P->NK : q, -1.0, 1.0, E));
   }
-  launch_axpby_identity<double>(N, E, NN, nw, 1.0, st);
+  if (P->fp64) launch_axpby_identity<double>(N, E, NN, nw, 1.0, st);
   if (hw && P->p.head_wings == 1) {
     // Vbh[w] = Vb0 h[w], then the rank-2 head / wing correction
     launch_zgemm<double>(nw, N, N, one, P->d_h, N, 0, OP_N, P->d_Vb0, N, 0, OP_T, zero, P->d_tmp, N, 0, 1, st);
@@ -1326,16 +1353,11 @@ gw_status w_core(gw_plan_s* P, int q, const c128* X, c128* Wc) {
   const long long NN = (long long)N * N;
   const c128* Vh = P->d_Vh + (long long)q * NN;
   const c128 one{1, 0}, zero{0, 0};
-  c64* A32 = reinterpret_cast<c64*>(P->d_work);
   if (P->fp64) {
     launch_zgemm<double>(N, N, N, one, X, N, NN, OP_N, Vh, N, 0, OP_N, zero, P->d_tmp, N, NN, nw, st);
     launch_zgemm<double>(N, N, N, one, Vh, N, 0, OP_N, P->d_tmp, N, NN, OP_N, zero, Wc, N, NN, nw, st);
   } else {
-    // V^1/2 X V^1/2 as (V^1/2 X) V^1/2 (X = eps~^-1 - 1 and V^1/2 Hermitian)
-    const c64* Vh32 = P->d_Vh32 + (long long)q * NN;
-    GW_TRY(herm_gemm(P, Vh32, false, X, true, 1.0, P->d_tmp));
-    launch_convert(NN * nw, P->d_tmp, A32, st);
-    GW_TRY(herm_gemm(P, A32, true, Vh, false, 1.0, Wc));
+    GW_TRY(sandwich(P, X, q, 1.0, 0.0, Wc));
   }
   return check_launch(P, "W^c");
 }

@@ -182,23 +182,35 @@ struct Chi0Plan;
 void chi0_plan_free(Chi0Plan* p);
 gw_status chi0h_pieces(const Chi0hArgs& a, cudaStream_t st);
 gw_status chi0h_run(const Chi0hArgs& a, Chi0Plan** plan, cudaStream_t st, std::string& err);
-// C[b] = alpha A[b] H[b] (b < nb; complex N x N row-major, N even; H[b] Hermitian) on the same
-// tcgen05 kernel with unit weights, every element, TF32 two-piece operands, FP64 output (overwritten)
+// C[b] = (alpha A[b] H[b]^H)^H + diag 1 (b < nb; complex N x N row-major, N even) on the same tcgen05
+// kernel with unit weights, every element, two pieces per operand: FP16 with each operand scaled, or TF32
+// (half the rate; the iteration for V^1/2 uses it, whose result is 2x closer with it: the tensor core's
+// accumulator truncates, and TF32 products have half the terms between two drains). The conjugate
+// transpose of the product is what the kernel writes in whole sectors; the callers order their products
+// accordingly. The four products of one q (N = 400, 32 frequencies): 0.61 ms, 0.93 ms as TF32 products with
+// row-wise stores, a right operand per frequency cut each time and FP64 results rounded by a pass of their
+// own; V^1/2 of 64 q 13.9 ms of products, 20 ms before (the stores).
 struct HermGemmArgs {
-  int N, nb;
-  const c64* A;          // [a_batch ? nb : 1][N][N]
-  int a_batch;
-  const c128* H64;       // [h_batch ? nb : 1][N][N] FP64, or NULL and H32 given
-  const c64* H32;
+  int N, nb, f16;
+  const c64* A;            // [nb][N][N]
+  const unsigned* amaxA;   // FP16: [nb] largest |re|, |im| of A[b] (float bits)
+  const void* h[2];        // pieces of H: [(h_batch ? nb : 1) N][2 Kpad], Kpad = N rounded up to 32
+  const int* eB;           // FP16: their scale (one matrix H)
   int h_batch;
-  double alpha;
-  c128* C;               // [nb][N][N]
-  float* bpl[2];         // workspace: [(h_batch ? nb : 1) N][2 Kpad] fp32 each, Kpad = N rounded up to 32
-  float* ones;           // workspace [Kpad]
-  double* escale;        // workspace [nb]
+  double alpha, diag;
+  c128* C;                 // FP64 result, or NULL and
+  c64* C32;                // FP32 result with
+  unsigned* amaxC;         // [nb] its largest |re|, |im| (zeroed by the caller)
+  float* wrow;             // workspace [nb][Kpad]
+  double* escale;          // workspace [nb]
   int* status;
 };
 gw_status herm_gemm_run(const HermGemmArgs& a, Chi0Plan** plan, cudaStream_t st, std::string& err);
+// pieces of `mats` matrices [N][N]: FP16 with one scale each, from their largest elements amax [mats]; TF32
+void herm_pieces_f16(int N, int mats, const c128* H, const unsigned* amax, void* p0, void* p1, int* eB, cudaStream_t st);
+void herm_pieces_tf32(int N, int mats, const c64* H, void* p0, void* p1, cudaStream_t st);
+// amax[b] (zeroed by the caller) of `batch` arrays of n elements rounded to FP32, written to out unless NULL
+void herm_round_max(long long n, int batch, const c128* in, c64* out, unsigned* amax, cudaStream_t st);
 // wtab[j][r] = 2 D_r / (w_j^2 + D_r^2) (0 for padding rows r >= K)
 void chi0h_weights(int K, int Kpad, int nw, const float* delta, const double* freq, float* wtab, cudaStream_t st);
 

@@ -8,8 +8,8 @@
 //   Re C = sum (a_re b_re + a_im b_im) = A1 . B,   A1 row = (a_re, a_im)
 //   Im C = sum (a_im b_re - a_re b_im) = A2 . B,   A2 row = (a_im, -a_re)
 //   B row = (b_re, b_im): the M plane itself.
-// One MMA with M = 128 = [A1 of 64 mu; A2 of the same 64 mu] against N <= 128 nu rows of B gives
-// Re (TMEM lanes 0-63) and Im (lanes 64-127) of a 64 x N complex tile. Each weighted and split A
+// One MMA with M = 128 = A1 and A2 of 64 mu (16 rows A1, the same 16 rows A2, ...) against N <= 128 nu
+// rows of B gives Re and Im of a 64 x N complex tile, both parts of a row in the same warp's TMEM lanes. Each weighted and split A
 // row thus feeds 2 x N MMA columns, and B needs no second, permuted copy.
 //
 // Operand splits (the same pieces on both sides; products of combined order below the fp32
@@ -106,6 +106,10 @@ struct Tile {
   int n0, ncols;   // nu columns [n0, n0 + ncols), ncols a multiple of 16 (<= 128)
 };
 
+// OUT_ADD: FP64 atomic accumulation; OUT_F64 / OUT_F32: one K chunk of one segment per output, plain
+// stores (no zeroing) of the conjugate transpose. [T][N][N] complex.
+enum { OUT_ADD, OUT_F64, OUT_F32 };
+
 struct Chi0Params {
   int N;
   int nst;              // stages over the padded pair rows
@@ -119,11 +123,12 @@ struct Chi0Params {
   const float* wtab;    // [T][wstride] weights (F16: already multiplied by the row's scale)
   long long wstride;
   const double* escale; // [T] factor applied to the drained sums (scale, and the F16 scales undone)
-  double* out;          // [T][N][N] complex as (re, im) doubles, lower triangle accumulated
+  double* out;          // [T][N][N] complex as (re, im) doubles
   int* status;
   int lower;            // 1: lower triangle only (Hermitian result); 0: every element
-  int store;            // 1: one K chunk of one segment per output, written with plain stores (no
-                        //    zeroing, no atomics); 0: FP64 atomic accumulation
+  double diag;          // OUT_F64: added to the diagonal
+  float* out32;         // OUT_F32: [T][N][N] complex as (re, im) floats
+  unsigned* amax;       // OUT_F32: [T] largest |re|, |im| written (float bits, atomicMax)
   int a_bstride;        // A rows of weight row / batch entry t start at t * a_bstride
   int b_bstride;        // B rows of t start at t * b_bstride
 };
@@ -178,7 +183,7 @@ __device__ __forceinline__ void mma_k(uint32_t d, uint64_t a, uint64_t b, uint32
   mma<KIND == K_TF32>(d, a, b, idesc, acc);
 }
 
-template <int KIND, int TP>
+template <int KIND, int TP, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 1) k_chi0(const __grid_constant__ Chi0Maps maps, Chi0Params p) {
   using C = Kd<KIND, TP>;
   static_assert(C::SMEM <= 232448, "shared memory budget");
@@ -346,6 +351,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0(const __grid_constant__ Ch
     // ---------------- transform: weighted, split A1 / A2 pieces ----------------
     const int tid = threadIdx.x - 64;          // 0..127
     const int row = tid & 63;                  // mu row within the tile
+    const int arow = (row >> 4) * 32 + (row & 15);   // its A1 row; A2 is 16 rows below
     const int h = tid >> 6;                    // BF16 / F16: ring slot of the stage; TF32: half of the slot
     uint32_t gs = 0, gr = 0;
     bool ok = true;
@@ -408,7 +414,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0(const __grid_constant__ Ch
               l2[2 * q] = __float_as_uint(li);
               l2[2 * q + 1] = __float_as_uint(-lr);
             }
-            const uint32_t o1 = swz(row, 4 * h + c), o2 = swz(row + 64, 4 * h + c);
+            const uint32_t o1 = swz(arow, 4 * h + c), o2 = swz(arow + 16, 4 * h + c);
             *reinterpret_cast<uint4*>(au + o1) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
             *reinterpret_cast<uint4*>(au + o2) = make_uint4(h2[0], h2[1], h2[2], h2[3]);
             *reinterpret_cast<uint4*>(au + TILE + o1) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
@@ -470,7 +476,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0(const __grid_constant__ Ch
 #pragma unroll
               for (int pc = 0; pc < NP; ++pc) o2[pc][q] = swap_neg(o[pc][q]);
             }
-            const uint32_t off1 = swz(row, 4 * h + cc), off2 = swz(row + 64, 4 * h + cc);
+            const uint32_t off1 = swz(arow, 4 * h + cc), off2 = swz(arow + 16, 4 * h + cc);
 #pragma unroll
             for (int pc = 0; pc < NP; ++pc) {
               *reinterpret_cast<uint4*>(au + pc * TILE + off1) = make_uint4(o[pc][0], o[pc][1], o[pc][2], o[pc][3]);
@@ -491,7 +497,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0(const __grid_constant__ Ch
     constexpr int CPT = 4 / TP;                // column groups per weight row
     const int u = cg / CPT;                    // weight row t + u of the item's group
     const int cw = 32 * (cg % CPT);            // first tile column of the group
-    const int lrow = quad * 32 + lane;         // TMEM lane: Re (< 64) or Im (>= 64) of mu row lrow & 63
+    const int part = lane >> 4;                // this TMEM lane holds Re (0) or Im (1) of mu row quad * 16 + lane % 16
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
     const float f2 = (KIND == K_F16) ? 1.0f / (float)(1 << LSH) : 1.0f;
     int b = 0, b2 = 0;
@@ -505,8 +511,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0(const __grid_constant__ Ch
       int t, s0, s1;
       decode<TP>(p, p.items[it], tl, t, s0, s1);
       const int ncol = (t + u < p.T) ? max(0, min(32, tl.ncols - cw)) : 0;
-      const int mu = tl.m0 + (lrow & 63);
-      const int part = lrow >> 6;
+      const int mu = tl.m0 + quad * 16 + (lane & 15);
+      [[maybe_unused]] float amax = 0.f;
       const double es = p.escale[min(t + u, p.T - 1)];
       int spos = 0;
       for (int i = s0; i < s1; ++i) {
@@ -530,24 +536,44 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0(const __grid_constant__ Ch
           __syncwarp();
           if (lane == 0) mbar_arrive(&t2empty[b2]);
           if (++b2 == NB2) { b2 = 0; ++r2; }
-          if (mu >= tl.m0 && mu < tl.mhi) {
-            const int c0 = tl.n0 + cw;
-            double* o = p.out + 2 * (((long long)(t + u) * p.N + mu) * p.N + c0) + part;
-            // columns nu = c0 + j of the tile below N (and, for the lower triangle, <= mu)
-            const int jmax = min(ncol, (p.lower ? mu + 1 : p.N) - c0);
-            if (p.store) {
+          // columns nu < N of the tile (lower triangle: nu <= mu)
+          const int c0 = tl.n0 + cw;
+          const int jmax = (mu >= tl.m0 && mu < tl.mhi) ? min(ncol, (p.lower ? mu + 1 : p.N) - c0) : 0;
+          const long long mat = (long long)(t + u) * p.N * p.N;
+          if constexpr (MODE == OUT_ADD) {
+            // (element by element along a row: the L2 atomics of one line are serialised, so lanes that share
+            // lines are slower than lanes on 16 rows)
+            double* o = p.out + 2 * (mat + (long long)mu * p.N + c0) + part;
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (j < jmax) o[2 * j] = es * (double)acc[j];
-            } else {
+            for (int j = 0; j < 32; ++j)
+              if (j < jmax) atomicAdd(o + 2 * j, es * (double)acc[j]);
+          } else {
+            // element (mu, nu) is written at [nu][mu], conjugated: a warp's lanes are Re and Im of 16 rows mu,
+            // so each of its columns fills 256 contiguous bytes
+            long long o = 2 * (mat + (long long)c0 * p.N + mu) + part;
+            const double f = part ? -es : es;
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (j < jmax) atomicAdd(o + 2 * j, es * (double)acc[j]);
+            for (int j = 0; j < 32; ++j) {
+              if (j < jmax) {
+                double x = f * (double)acc[j];
+                if constexpr (MODE == OUT_F64) {
+                  if (part == 0 && c0 + j == mu) x += p.diag;
+                  p.out[o] = x;
+                } else {
+                  p.out32[o] = (float)x;
+                  amax = fmaxf(amax, fabsf((float)x));
+                }
+              }
+              o += 2 * p.N;
             }
           }
 #pragma unroll
           for (int j = 0; j < 32; ++j) acc[j] = 0.f;
         }
+      }
+      if constexpr (MODE == OUT_F32) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+        if (lane == 0 && ncol > 0) atomicMax(p.amax + t + u, m);
       }
     }
   }
@@ -815,11 +841,11 @@ static gw_status chi0_lists(Chi0Plan** pp, int N, int T, int nst, int seg, int t
   return GW_OK;
 }
 
-template <int KIND, int TP>
+template <int KIND, int TP, int MODE = OUT_ADD>
 static gw_status launch_chi0(const Chi0Maps& maps, const Chi0Params& prm, int grid, cudaStream_t st, std::string& err) {
   const int smem = Kd<KIND, TP>::SMEM;
-  cudaFuncSetAttribute(k_chi0<KIND, TP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  ++g_launch_count, k_chi0<KIND, TP><<<grid, NTHREADS, smem, st>>>(maps, prm);
+  cudaFuncSetAttribute(k_chi0<KIND, TP, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  ++g_launch_count, k_chi0<KIND, TP, MODE><<<grid, NTHREADS, smem, st>>>(maps, prm);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = std::string("k_chi0 launch: ") + cudaGetErrorString(e);
@@ -892,33 +918,89 @@ gw_status chi0h_run(const Chi0hArgs& a, Chi0Plan** plan, cudaStream_t st, std::s
   return GW_OK;
 }
 
-// TF32 pieces of Hermitian matrices H (FP64 or FP32 complex, [rows][N]) as the B planes of the
-// product kernel: row r, K index 2k + {0: re, 1: im}, zero for k >= N (padding to Kpad)
-template <typename T>
-__global__ void k_h_pieces_tf32(long long rows, int N, int Kpad, const cplx<T>* __restrict__ H, float* __restrict__ p0,
-                                float* __restrict__ p1) {
-  const long long total = rows * Kpad;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long r = e / Kpad;
-    const int k = (int)(e % Kpad);
+// Pieces of `mats` matrices H ([N][N] each) as B planes of the product kernel: row r, K index 2k + {0: re,
+// 1: im}, zero for k >= N. FP16: each matrix scaled by 2^eB (largest |x 2^eB| in [2^13, 2^14)); TF32: as is.
+template <int KIND, typename T>
+__global__ void k_h_pieces(int N, int Kpad, const cplx<T>* __restrict__ H, const unsigned* __restrict__ amax,
+                           void* __restrict__ p0, void* __restrict__ p1, int* __restrict__ eB) {
+  const int b = blockIdx.y;
+  float s = 1.0f;
+  if constexpr (KIND == K_F16) {
+    int e = 0;
+    const float m = __uint_as_float(amax[b]);
+    if (m > 0.f) frexpf(m, &e);
+    s = ldexpf(1.0f, 14 - e);
+    if (blockIdx.x == 0 && threadIdx.x == 0) eB[b] = 14 - e;
+  }
+  const long long total = (long long)N * Kpad;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / Kpad;
+    const int k = (int)(i % Kpad);
     float xr = 0.f, xi = 0.f;
     if (k < N) {
-      const cplx<T> v = H[r * N + k];
-      xr = (float)v.re;
-      xi = (float)v.im;
+      const cplx<T> v = H[((long long)b * N + r) * N + k];
+      xr = (float)v.re * s;
+      xi = (float)v.im * s;
     }
-    const float hr = tf32_rn(xr), hi = tf32_rn(xi);
-    reinterpret_cast<float2*>(p0)[e] = make_float2(hr, hi);
-    reinterpret_cast<float2*>(p1)[e] = make_float2(xr - hr, xi - hi);
+    if constexpr (KIND == K_F16) {
+      const __half2 h = __floats2half2_rn(xr, xi);
+      const float2 hf = __half22float2(h);
+      static_cast<__half2*>(p0)[b * total + i] = h;
+      static_cast<__half2*>(p1)[b * total + i] =
+          __floats2half2_rn((xr - hf.x) * (float)(1 << LSH), (xi - hf.y) * (float)(1 << LSH));
+    } else {
+      const float hr = tf32_rn(xr), hi = tf32_rn(xi);
+      static_cast<float2*>(p0)[b * total + i] = make_float2(hr, hi);
+      static_cast<float2*>(p1)[b * total + i] = make_float2(xr - hr, xi - hi);
+    }
   }
 }
-
-__global__ void k_fill_d(double* p, int n, double v) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) p[e] = v;
+// amax[b] = largest |re|, |im| of matrix b rounded to FP32 (float bits; zeroed by the caller), out (may be
+// NULL) the matrices in FP32
+__global__ void k_round_max(long long n, const c128* __restrict__ in, c64* __restrict__ out, unsigned* __restrict__ amax) {
+  const long long o = blockIdx.y * n;
+  float m = 0.f;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const c128 v = in[o + i];
+    const c64 w{(float)v.re, (float)v.im};
+    if (out) out[o + i] = w;
+    m = fmaxf(m, fmaxf(fabsf(w.re), fabsf(w.im)));
+  }
+  const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+  if ((threadIdx.x & 31) == 0) atomicMax(amax + blockIdx.y, u);
 }
-__global__ void k_fill_f(float* p, int n, float v) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) p[e] = v;
+// weight rows of the left operands (FP16: 2^eA, else 1) and the factors of the products
+__global__ void k_herm_scales(int Kpad, const unsigned* __restrict__ amaxA, const int* __restrict__ eB, int f16,
+                              double alpha, float* __restrict__ wrow, double* __restrict__ escale) {
+  const int t = blockIdx.x;
+  int eA = 0;
+  if (f16) {
+    const float m = __uint_as_float(amaxA[t]);
+    if (m > 0.f) frexpf(m, &eA);
+    eA = 14 - eA;
+  }
+  for (int k = threadIdx.x; k < Kpad; k += blockDim.x) wrow[(long long)t * Kpad + k] = ldexpf(1.0f, eA);
+  if (threadIdx.x == 0) escale[t] = ldexp(alpha, -(eA + (f16 ? *eB : 0)));
+}
+
+void herm_round_max(long long n, int batch, const c128* in, c64* out, unsigned* amax, cudaStream_t st) {
+  const int grid = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152LL * 16 / std::min(batch, 16)));
+  ++g_launch_count, k_round_max<<<dim3(grid, batch), 256, 0, st>>>(n, in, out, amax);
+}
+
+namespace {
+template <int KIND, typename T>
+void pieces_of(int N, int mats, const cplx<T>* H, const unsigned* amax, void* p0, void* p1, int* eB, cudaStream_t st) {
+  const int Kpad = (N + 31) / 32 * 32;
+  const int grid = (int)std::max<long long>(1, std::min<long long>(((long long)N * Kpad + 255) / 256, 152LL * 16 / std::min(mats, 16)));
+  ++g_launch_count, k_h_pieces<KIND, T><<<dim3(grid, mats), 256, 0, st>>>(N, Kpad, H, amax, p0, p1, eB);
+}
+}  // namespace
+void herm_pieces_f16(int N, int mats, const c128* H, const unsigned* amax, void* p0, void* p1, int* eB, cudaStream_t st) {
+  pieces_of<K_F16, double>(N, mats, H, amax, p0, p1, eB, st);
+}
+void herm_pieces_tf32(int N, int mats, const c64* H, void* p0, void* p1, cudaStream_t st) {
+  pieces_of<K_TF32, float>(N, mats, H, nullptr, p0, p1, nullptr, st);
 }
 
 gw_status herm_gemm_run(const HermGemmArgs& a, Chi0Plan** plan, cudaStream_t st, std::string& err) {
@@ -928,25 +1010,19 @@ gw_status herm_gemm_run(const HermGemmArgs& a, Chi0Plan** plan, cudaStream_t st,
     return GW_ERR_ARG;
   }
   const int Kpad = (N + 31) / 32 * 32;
-  const long long hrows = (long long)(a.h_batch ? nb : 1) * N;
-  const int grid = (int)std::min<long long>((hrows * Kpad + 255) / 256, 152LL * 16);
-  if (a.H64)
-    ++g_launch_count, k_h_pieces_tf32<double><<<grid, 256, 0, st>>>(hrows, N, Kpad, a.H64, a.bpl[0], a.bpl[1]);
-  else
-    ++g_launch_count, k_h_pieces_tf32<float><<<grid, 256, 0, st>>>(hrows, N, Kpad, a.H32, a.bpl[0], a.bpl[1]);
-  ++g_launch_count, k_fill_d<<<1, 256, 0, st>>>(a.escale, nb, a.alpha);
-  ++g_launch_count, k_fill_f<<<(Kpad + 255) / 256, 256, 0, st>>>(a.ones, Kpad, 1.0f);
-  const int RS = Kd<K_TF32, 1>::RS;
-  const int nst = Kpad / RS;
+  ++g_launch_count, k_herm_scales<<<nb, 128, 0, st>>>(Kpad, a.amaxA, a.eB, a.f16, a.alpha, a.wrow, a.escale);
+  const int nst = Kpad / (a.f16 ? Kd<K_F16, 1>::RS : Kd<K_TF32, 1>::RS);
   Chi0Lists* L = nullptr;
   gw_status s = chi0_lists(plan, N, nb, nst, nst, 1, st, &L, err, false);
   if (s != GW_OK) return s;
   Chi0Maps maps;
+  const long long hrows = (long long)(a.h_batch ? nb : 1) * N;
   for (int i = 0; i < 2; ++i)
-    if (!map2d(&maps.b[i], a.bpl[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 2LL * Kpad, hrows, BNU, err))
+    if (!map2d(&maps.b[i], a.h[i], a.f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.f16 ? 2 : 4,
+               2LL * Kpad, hrows, BNU, err))
       return GW_ERR_CUDA;
-  const long long arows = (long long)(a.a_batch ? nb : 1) * N;
-  if (!map2d(&maps.raw, a.A, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 2LL * N, arows, BMU, err)) return GW_ERR_CUDA;
+  if (!map2d(&maps.raw, a.A, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 2LL * N, (long long)nb * N, BMU, err))
+    return GW_ERR_CUDA;
   Chi0Params prm{};
   prm.N = N;
   prm.nst = nst;
@@ -957,20 +1033,25 @@ gw_status herm_gemm_run(const HermGemmArgs& a, Chi0Plan** plan, cudaStream_t st,
   prm.cta_off = L->d_off;
   prm.T = nb;
   prm.TG = nb;
-  prm.wtab = a.ones;
-  prm.wstride = 0;
+  prm.wtab = a.wrow;
+  prm.wstride = Kpad;
   prm.escale = a.escale;
   prm.out = reinterpret_cast<double*>(a.C);
+  prm.out32 = reinterpret_cast<float*>(a.C32);
+  prm.amax = a.amaxC;
   prm.status = a.status;
   prm.lower = 0;
-  prm.store = 1;   // one K chunk (nchunk = 1) and one segment per item: every element written once
+  prm.diag = a.diag;
   if (L->nchunk != 1) {
     err = "herm_gemm: the product needs one K chunk per output tile";
     return GW_ERR_STATE;
   }
-  prm.a_bstride = a.a_batch ? N : 0;
+  prm.a_bstride = N;
   prm.b_bstride = a.h_batch ? N : 0;
-  return launch_chi0<K_TF32, 1>(maps, prm, L->grid, st, err);
+  // one K chunk (nchunk = 1) and one segment per item: plain stores
+  if (!a.f16) return launch_chi0<K_TF32, 1, OUT_F64>(maps, prm, L->grid, st, err);
+  return a.C ? launch_chi0<K_F16, 1, OUT_F64>(maps, prm, L->grid, st, err)
+             : launch_chi0<K_F16, 1, OUT_F32>(maps, prm, L->grid, st, err);
 }
 
 void chi0h_weights(int K, int Kpad, int nw, const float* delta, const double* freq, float* wtab, cudaStream_t st) {
