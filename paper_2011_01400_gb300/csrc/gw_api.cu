@@ -124,10 +124,14 @@ __global__ void k_trs_check(int n1, int n2, int n3, int NBd, const double* __res
     dv = fmax(dv, fmax(fabs(a.re - b.re), fabs(a.im + b.im)));
     av = fmax(av, fmax(fabs(a.re), fabs(a.im)));
   }
-  atomicMax(out, (unsigned long long)__double_as_longlong(de));
-  atomicMax(out + 1, (unsigned long long)__double_as_longlong(ae));
-  atomicMax(out + 2, (unsigned long long)__double_as_longlong(dv));
-  atomicMax(out + 3, (unsigned long long)__double_as_longlong(av));
+  // non-negative doubles order like their bit patterns; one atomic per warp and value
+  const double m[4] = {de, ae, dv, av};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    double x = m[i];
+    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+    if ((threadIdx.x & 31) == 0 && x > 0.0) atomicMax(out + i, (unsigned long long)__double_as_longlong(x));
+  }
 }
 
 // Y = V / c (typed), Z = I
@@ -924,7 +928,7 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
     unsigned long long* d_chk = nullptr;
     if ((s = dalloc(P, &d_chk, 4)) != GW_OK) return cleanup(s);
     CK(cudaMemsetAsync(d_chk, 0, 4 * sizeof(unsigned long long), st));
-    ++g_launch_count, k_trs_check<<<152 * 8, 256, 0, st>>>(prob->nk[0], prob->nk[1], prob->nk[2], P->NBd, prob->eps, N,
+    ++g_launch_count, k_trs_check<<<(int)std::min<size_t>(152 * 4, (NN * P->NK + 1023) / 1024), 256, 0, st>>>(prob->nk[0], prob->nk[1], prob->nk[2], P->NBd, prob->eps, N,
                                                             reinterpret_cast<const c128*>(prob->V), d_chk);
     unsigned long long h[4] = {0, 0, 0, 0};
     CK(cudaMemcpyAsync(h, d_chk, sizeof(h), cudaMemcpyDeviceToHost, st));
@@ -1085,7 +1089,7 @@ gw_status chi0_prepare(gw_plan_s* P, const int* qs, int nq) {
     }
   }
   launch_wnorm(nw, nq, P->d_wG, P->d_wn, st);
-  launch_small_jacobi(nw, nq, P->d_wG, P->d_wlam, P->d_wU, st);
+  launch_small_jacobi(nw, nq, P->d_wG, P->d_wlam, P->d_wU, st, true);
   launch_wproj(nw, nq, P->d_wU, P->d_wn, P->d_wE, P->d_wP, st);
   const long long sE = (long long)nw * (nw + 1);
   GW_CUDA(cudaMemsetAsync(P->d_werr, 0, sizeof(double) * sE * nq, st));
@@ -1179,7 +1183,7 @@ gw_status chi0_core(gw_plan_s* P, int q, c128* chi0) {
       launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), evec, q, kk0, nkk, MAP_K_IS_KK,
                           P->nocc, na, 0, nb, M, 1, P->ldm, st);
       GW_CUDA(cudaEventRecord(e0, st));
-      launch_chi0_simt<double>(N, K, M, P->ldm, nullptr, P->d_delta, P->d_freq, nw, scale, chi0, st);
+      launch_chi0_simt(N, K, M, P->ldm, P->d_delta, P->d_freq, nw, scale, chi0, st);
       GW_CUDA(cudaEventRecord(e1, st));
       // one direction (head_wings = 1) or the three Cartesian components for the average
       if (hw && !hw_avg)
@@ -1317,7 +1321,7 @@ gw_status eps_core(gw_plan_s* P, int q, const c128* chi0, c128* E) {
   if (P->fp64) launch_axpby_identity<double>(N, E, NN, nw, 1.0, st);
   if (hw && P->p.head_wings == 1) {
     // Vbh[w] = Vb0 h[w], then the rank-2 head / wing correction
-    launch_zgemm<double>(nw, N, N, one, P->d_h, N, 0, OP_N, P->d_Vb0, N, 0, OP_T, zero, P->d_tmp, N, 0, 1, st);
+    launch_row_dots(N, nw, N, 1.0, P->d_Vb0, 0, P->d_h, 0, P->d_tmp, 0, 1, N, 1, st);
     const double c = (P->p.spin / P->NK) * std::sqrt(4.0 * M_PI / P->p.omega_cell);
     launch_q0_correction(N, nw, E, P->d_x1, P->d_tmp, P->d_head, c, st);
   }
@@ -1337,10 +1341,8 @@ gw_status q0_average(gw_plan_s* P, c128* X) {
   const int N = P->N, nw = P->nw;
   const long long NN = (long long)N * N;
   const double c = (P->p.spin / P->NK) * std::sqrt(4.0 * M_PI / P->p.omega_cell);
-  launch_zgemm<double>(3 * nw, N, N, c128{-c, 0}, P->d_h3, N, 0, OP_N, P->d_Vb0, N, 0, OP_T, c128{0, 0}, P->d_Y3, N,
-                       0, 1, st);
-  launch_zgemm<double>(N, 3, N, c128{1, 0}, X, N, NN, OP_N, P->d_Y3, N, 3LL * N, OP_T, c128{0, 0}, P->d_G3, 3,
-                       3LL * N, nw, st);
+  launch_row_dots(N, 3 * nw, N, -c, P->d_Vb0, 0, P->d_h3, 0, P->d_Y3, 0, 1, N, 1, st);
+  launch_row_dots(N, 3, N, 1.0, X, NN, P->d_Y3, 3LL * N, P->d_G3, 3LL * N, 3, 1, nw, st);
   launch_q0avg_moments(N, nw, P->d_Y3, P->d_G3, P->d_A6, P->d_dirs, P->n_dirs, P->d_m10, P->d_status, st);
   launch_q0avg_update(N, nw, X, NN, P->d_x1, P->d_G3, P->d_m10, st);
   return check_launch(P, "q = 0 direction average");

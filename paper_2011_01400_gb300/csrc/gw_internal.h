@@ -81,10 +81,12 @@ template <typename T>
 void launch_zgemm(int m, int n, int k, cplx<T> alpha, const cplx<T>* A, long long lda, long long sA, Op opA,
                   const cplx<T>* B, long long ldb, long long sB, Op opB, cplx<T> beta, cplx<T>* C,
                   long long ldc, long long sC, int batch, cudaStream_t st);
-// chi0[w][mu][nu] += scale * sum_r w_w(D_r) Mt[mu][r] conj(Mt[nu][r]),  Mt row-major [N][ldm]
-template <typename T>
-void launch_chi0_simt(int N, int K, const cplx<T>* Mt, long long ldm, const float* delta_f, const double* delta_d,
-                      const double* freq, int nw, double scale, c128* chi0, cudaStream_t st);
+// chi0[w][mu][nu] += scale * sum_r w_w(D_r) Mt[mu][r] conj(Mt[nu][r]),  Mt row-major [N][ldm] (FP64)
+void launch_chi0_simt(int N, int K, const c128* Mt, long long ldm, const double* delta, const double* freq, int nw,
+                      double scale, c128* chi0, cudaStream_t st);
+// out[b so + r sr + c sc] = alpha sum_k A[b sA + r K + k] B[b sB + c K + k]
+void launch_row_dots(int rows, int cols, int K, double alpha, const c128* A, long long sA, const c128* B, long long sB,
+                     c128* out, long long so, long long sr, long long sc, int batch, cudaStream_t st);
 // k_inv.cu: per matrix b: A[b] (Hermitian PD, row-major N x N, FP64; its upper triangle is read)
 // -> A[b] := A[b]^{-1} - I. Sets ST_NOT_PD. work: inv_work_bytes(N, batch) bytes, 16-byte aligned.
 size_t inv_work_bytes(int N, int batch);
@@ -216,7 +218,8 @@ void chi0h_weights(int K, int Kpad, int nw, const float* delta, const double* fr
 
 // Ritz modes and the surrogate reconstruction (k_modes.cu); small sizes nb <= 64
 void launch_small_chol_linv(int nb, int batch, const c128* G, c128* Linv, int* status, cudaStream_t st);
-void launch_small_jacobi(int nb, int batch, const c128* H, double* theta, c128* Z, cudaStream_t st);
+// real: H has no imaginary part (not read)
+void launch_small_jacobi(int nb, int batch, const c128* H, double* theta, c128* Z, cudaStream_t st, bool real = false);
 void launch_mode_diag(int N, int k, int nc, const c128* U, const c128* T, long long sT, float* d, int ldd, int c0,
                       cudaStream_t st);
 void launch_sur_inputs(int rows, int nc, const float* d, float* x, float* sig, cudaStream_t st);
