@@ -239,10 +239,10 @@ gw_status gw_qp(gw_plan plan, int32_t sys, const gw_complex* sigma, const double
 
 /* gw_qp without any device allocation (the paper has no counterpart: a deployment variant).
  * Same arguments, arithmetic and results as gw_qp; the per-(k, n) QP energies and Newton flags
- * live in one fixed file-scope device array of GW_QP_STATIC_MAX pairs instead of a
- * cudaMalloc/cudaFree pair per call. For callers that cannot allocate device memory when
- * they solve the QP equation: a process whose device memory is held by a caching allocator,
- * or a serving loop that must not take the device-wide synchronisation of cudaFree.
+ * live in one fixed file-scope device array of GW_QP_STATIC_MAX pairs instead of the plan's
+ * workspace. For callers that cannot allocate device memory when they solve the QP equation: a
+ * process whose device memory is held by a caching allocator, or a serving loop that must not
+ * take a device-wide synchronisation.
  * The plan itself still owns the workspace gw_plan_create allocated.
  * - N_k * (sigma_hi - sigma_lo) > GW_QP_STATIC_MAX: GW_ERR_ARG, nothing launched (use gw_qp).
  * - The current CUDA device must be the plan's device (the one current at gw_plan_create):

@@ -205,6 +205,9 @@ struct gw_plan_s {
   int err = 0;              // sticky error
   int chi0_q = -1, wc_q = -1;
   // device memory owned by the plan
+  uint8_t* arena = nullptr;         // one cudaMalloc for the buffers of gw_plan_create
+  size_t arena_size = 0, arena_used = 0, arena_need = 0;
+  bool measuring = false;           // dalloc only adds up arena_need
   std::vector<void*> allocs;
   std::vector<size_t> alloc_bytes;  // size of each entry of allocs
   size_t ws_bytes = 0;              // sum of alloc_bytes
@@ -231,6 +234,9 @@ struct gw_plan_s {
   c128* d_tmp = nullptr;    // [nw][N][N]
   c128* d_sigma = nullptr;  // [NK][nsig][nw]
   double* d_head = nullptr; // [nw]
+  double* d_nsc = nullptr;  // [NK] norms of V(q) for the V^1/2 iteration
+  double* d_qp_e = nullptr; // gw_qp: energies and flags [NK][nsig]
+  int* d_qp_c = nullptr;
   c128* d_h = nullptr;      // [nw][N]
   // direction-averaged q = 0 (head_wings = 2)
   c128* d_pq3 = nullptr;    // [3][ldm] Cartesian components of p . q^
@@ -250,8 +256,7 @@ struct gw_plan_s {
   c128* d_pq = nullptr;       // [ldm]
   void* d_A = nullptr;        // sigma rows [R][N]
   void* d_Apl[2] = {};        // split precision: bf16 / tf32 pieces of the sigma rows [R][2*Kx]
-  double* d_Sx = nullptr;     // gw_sigma_x: S per row; FP32 rows A V [R][Kx] and V(q) in fp32
-  c64 *d_Ux = nullptr, *d_Vx32 = nullptr;
+  double* d_Sx = nullptr;     // gw_sigma_x: S per row (split path: per q of a group and column block)
   void* d_U = nullptr;        // [R][N]
   double* d_S_d = nullptr;    // [R][nw]
   float* d_S_f = nullptr;
@@ -337,13 +342,30 @@ struct gw_plan_s {
 
 namespace {
 
+// Device memory of a plan. The buffers of gw_plan_create are one cudaMalloc (plan_arena), cut here; what is
+// allocated later, or does not fit, is a cudaMalloc of its own.
+size_t arena_round(size_t bytes) { return (bytes + 1023) / 1024 * 1024; }
+
 template <typename T> gw_status dalloc(gw_plan_s* P, T** ptr, size_t count) {
   const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
+  if (P->measuring) {
+    P->arena_need += arena_round(bytes);
+    return GW_OK;
+  }
   if (P->ws_limit && P->ws_bytes + bytes > P->ws_limit)
     return fail(GW_ERR_NOMEM, "workspace limit GW_WORKSPACE_LIMIT = " + std::to_string(P->ws_limit) +
                                   " bytes reached: " + std::to_string(P->ws_bytes) + " held, " +
                                   std::to_string(bytes) + " more requested");
   void* p = nullptr;
+  if (P->arena_used + arena_round(bytes) <= P->arena_size) {
+    p = P->arena + P->arena_used;
+    P->arena_used += arena_round(bytes);
+    P->allocs.push_back(p);
+    P->alloc_bytes.push_back(bytes);
+    P->ws_bytes += bytes;
+    *ptr = static_cast<T*>(p);
+    return GW_OK;
+  }
   ++g_alloc_count;
   cudaError_t e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
@@ -358,9 +380,14 @@ template <typename T> gw_status dalloc(gw_plan_s* P, T** ptr, size_t count) {
   return GW_OK;
 }
 
+bool in_arena(const gw_plan_s* P, const void* p) {
+  return P->arena && p >= P->arena && p < P->arena + P->arena_size;
+}
+
 // frees the most recent dalloc
 void dfree_last(gw_plan_s* P) {
-  cudaFree(P->allocs.back());
+  if (in_arena(P, P->allocs.back())) P->arena_used -= arena_round(P->alloc_bytes.back());
+  else cudaFree(P->allocs.back());
   P->allocs.pop_back();
   P->ws_bytes -= P->alloc_bytes.back();
   P->alloc_bytes.pop_back();
@@ -463,22 +490,14 @@ gw_status newton_schulz_tc(gw_plan_s* P, c128* Vio, int batch, int iters) {
   const int N = P->N, nb = P->nw;
   const long long s = (long long)N * N;
   const size_t Kpad = (size_t)(N + 31) / 32 * 32;
-  double* d_c;
-  c64 *Y, *Yh, *Z, *Zh, *Tm, *Th;
-  c128* C;
-  float* pc[2];
-  unsigned* d_dev;
-  const size_t held = P->allocs.size();
-  GW_TRY(dalloc(P, &d_c, batch));
-  GW_TRY(dalloc(P, &Y, s * nb));
-  GW_TRY(dalloc(P, &Yh, s * nb));
-  GW_TRY(dalloc(P, &Z, s * nb));
-  GW_TRY(dalloc(P, &Zh, s * nb));
-  GW_TRY(dalloc(P, &Tm, s * nb));
-  GW_TRY(dalloc(P, &Th, s * nb));
-  GW_TRY(dalloc(P, &C, s * nb));
-  for (auto& p : pc) GW_TRY(dalloc(P, &p, (size_t)nb * N * 2 * Kpad));
-  GW_TRY(dalloc(P, &d_dev, 1));
+  // all on buffers of the plan that are not in use yet (each of nw N^2 c128; d_work holds the pieces)
+  double* d_c = P->d_nsc;
+  c64 *Y = reinterpret_cast<c64*>(P->d_chi0), *Yh = Y + s * nb;
+  c64 *Z = reinterpret_cast<c64*>(P->d_E), *Zh = Z + s * nb;
+  c64 *Tm = reinterpret_cast<c64*>(P->d_Wc), *Th = Tm + s * nb;
+  c128* C = P->d_tmp;
+  float* pc[2] = {reinterpret_cast<float*>(P->d_work), reinterpret_cast<float*>(P->d_work) + (size_t)nb * N * 2 * Kpad};
+  unsigned* d_dev = P->d_absmax;
   // X, X^H <- alpha A H + d 1, H given by its conjugate transpose Hh
   auto product = [&](const c64* A, const c64* Hh, double alpha, float d, c64* X, c64* XH, int n) -> gw_status {
     herm_pieces_tf32(N, n, Hh, pc[0], pc[1], P->st);
@@ -533,7 +552,6 @@ gw_status newton_schulz_tc(gw_plan_s* P, c128* Vio, int batch, int iters) {
   GW_TRY(check_launch(P, "newton_schulz"));
   cudaError_t e = cudaStreamSynchronize(P->st);
   if (e != cudaSuccess) return fail(GW_ERR_CUDA, std::string("newton_schulz: ") + cudaGetErrorString(e));
-  while (P->allocs.size() > held) dfree_last(P);
   return GW_OK;
 }
 
@@ -770,117 +788,144 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
   const int N = P->N, nw = P->nw;
   const size_t NN = (size_t)N * N;
   gw_status s;
-#define ALLOC(ptr, n)                                 \
-  do {                                                \
-    s = dalloc(P, &ptr, (n));                         \
-    if (s != GW_OK) return cleanup(s);                \
-  } while (0)
-  ALLOC(P->d_freq, nw);
-  ALLOC(P->d_fw, nw);
-  ALLOC(P->d_mu, 1);
-  ALLOC(P->d_status, 1);
-  ALLOC(P->d_Vh, NN * P->NK);
-  ALLOC(P->d_chi0, NN * nw);
-  ALLOC(P->d_E, NN * nw);
-  ALLOC(P->d_Wc, NN * nw);
-  ALLOC(P->d_work, std::max(NN * nw, (inv_work_bytes(N, nw) + sizeof(c128) - 1) / sizeof(c128)));
-  ALLOC(P->d_tmp, NN * nw);
-  ALLOC(P->d_sigma, (size_t)P->NK * P->nsig * nw);
-  ALLOC(P->d_head, nw);
-  ALLOC(P->d_h, (size_t)nw * N);
-  if (P->fp64) {
-    c128* t;
-    ALLOC(t, (size_t)toff);
-    P->d_T1 = t;
-  } else {
-    c64* t;
-    ALLOC(t, (size_t)toff);
-    P->d_T1 = t;
-  }
-  if (prob->head_wings) {
-    ALLOC(P->d_Vb0, NN);
-    ALLOC(P->d_x1, N);
-    ALLOC(P->d_v1, 1);
-  }
-  // chunk sizes: ~512 MB per M-type buffer
-  const size_t esz = P->fp64 ? sizeof(c128) : sizeof(c64);
-  const size_t budget = 512ull << 20;
-  const long long rows_chi = (long long)P->nocc * P->nunocc;
-  P->chi_nkk = (int)std::max<long long>(1, std::min<long long>(P->NK, budget / (rows_chi * N * esz)));
-  P->ldm = ((rows_chi * P->chi_nkk + 31) / 32) * 32;
-  const long long rows_sig = (long long)P->nsig * P->NBd;
-  P->sig_nkk = (int)std::max<long long>(1, std::min<long long>(P->NK, budget / (rows_sig * N * esz)));
-  P->sig_rows = rows_sig * P->sig_nkk;
-  if (P->fp64) {
-    c128 *a, *b, *c;
-    ALLOC(a, (size_t)N * P->ldm);
-    ALLOC(b, (size_t)P->sig_rows * N);
-    ALLOC(c, (size_t)P->sig_rows * N);
-    P->d_M = a;
-    P->d_A = b;
-    P->d_U = c;
-    ALLOC(P->d_S_d, (size_t)P->sig_rows * nw);
-  } else {
-    c64* b;
-    P->Kx = ((N + 31) / 32) * 32;
-    ALLOC(P->d_evec32, (size_t)P->NK * P->NB * P->NBd);
-    ALLOC(b, (size_t)P->sig_rows * P->Kx);   // raw plane of the Sigma rows, zero beyond n_aux
-    P->d_A = b;
-    ALLOC(P->d_S_f, (size_t)P->sig_rows * nw);
-    for (int i = 0; i < 2; ++i) {
-      uint8_t* pp;
-      ALLOC(pp, (size_t)P->sig_rows * 2 * P->Kx * (P->prec == GW_3XTF32 ? 4 : 2));
-      P->d_Apl[i] = pp;
+#define ALLOC(ptr, n) GW_TRY(dalloc(P, &ptr, (n)))
+  auto allocate = [&]() -> gw_status {
+    const size_t kp = (size_t)(N + 31) / 32 * 32;
+    ALLOC(P->d_freq, nw);
+    ALLOC(P->d_fw, nw);
+    ALLOC(P->d_mu, 1);
+    ALLOC(P->d_status, 1);
+    ALLOC(P->d_nsc, P->NK);
+    ALLOC(P->d_qp_e, (size_t)P->NK * P->nsig);
+    ALLOC(P->d_qp_c, (size_t)P->NK * P->nsig);
+    ALLOC(P->d_Vh, NN * P->NK);
+    ALLOC(P->d_chi0, NN * nw);
+    ALLOC(P->d_E, NN * nw);
+    ALLOC(P->d_Wc, NN * nw);
+    // (FP32 copies of two matrices per frequency, the workspace of nw inversions, the pieces of the V^1/2 iteration)
+    ALLOC(P->d_work, std::max({NN * nw, (inv_work_bytes(N, nw) + sizeof(c128) - 1) / sizeof(c128), (size_t)nw * N * kp}));
+    ALLOC(P->d_tmp, NN * nw);
+    ALLOC(P->d_sigma, (size_t)P->NK * P->nsig * nw);
+    ALLOC(P->d_head, nw);
+    ALLOC(P->d_h, (size_t)nw * N);
+    if (P->fp64) {
+      c128* t;
+      ALLOC(t, (size_t)toff);
+      P->d_T1 = t;
+    } else {
+      c64* t;
+      ALLOC(t, (size_t)toff);
+      P->d_T1 = t;
     }
-    const size_t we = (size_t)nw * N * 2 * P->Kx * (P->prec == GW_3XTF32 ? 4 : 2);
-    for (int i = 0; i < (P->prec == GW_3XTF32 ? 4 : 6); ++i) {
-      uint8_t* pp;
-      ALLOC(pp, we);
-      P->d_Wpl.b[i] = pp;
+    if (prob->head_wings) {
+      ALLOC(P->d_Vb0, NN);
+      ALLOC(P->d_x1, N);
+      ALLOC(P->d_v1, 1);
     }
-    const size_t vp = (size_t)(P->NK + (prob->head_wings ? 1 : 0)) * N;
-    for (auto& p : P->d_Vpc) ALLOC(p, vp * 2 * P->Kx);
-    ALLOC(P->d_Ve, vp / N);
+    // chunk sizes: ~512 MB per M-type buffer
+    const size_t esz = P->fp64 ? sizeof(c128) : sizeof(c64);
+    const size_t budget = 512ull << 20;
+    const long long rows_chi = (long long)P->nocc * P->nunocc;
+    P->chi_nkk = (int)std::max<long long>(1, std::min<long long>(P->NK, budget / (rows_chi * N * esz)));
+    P->ldm = ((rows_chi * P->chi_nkk + 31) / 32) * 32;
+    const long long rows_sig = (long long)P->nsig * P->NBd;
+    P->sig_nkk = (int)std::max<long long>(1, std::min<long long>(P->NK, budget / (rows_sig * N * esz)));
+    P->sig_rows = rows_sig * P->sig_nkk;
+    if (P->fp64) {
+      c128 *a, *b, *c;
+      ALLOC(a, (size_t)N * P->ldm);
+      ALLOC(b, (size_t)P->sig_rows * N);
+      ALLOC(c, (size_t)P->sig_rows * N);
+      P->d_M = a;
+      P->d_A = b;
+      P->d_U = c;
+      ALLOC(P->d_S_d, (size_t)P->sig_rows * nw);
+    } else {
+      c64* b;
+      P->Kx = ((N + 31) / 32) * 32;
+      ALLOC(P->d_evec32, (size_t)P->NK * P->NB * P->NBd);
+      ALLOC(b, (size_t)P->sig_rows * P->Kx);   // raw plane of the Sigma rows, zero beyond n_aux
+      P->d_A = b;
+      ALLOC(P->d_S_f, (size_t)P->sig_rows * nw);
+      for (int i = 0; i < 2; ++i) {
+        uint8_t* pp;
+        ALLOC(pp, (size_t)P->sig_rows * 2 * P->Kx * (P->prec == GW_3XTF32 ? 4 : 2));
+        P->d_Apl[i] = pp;
+      }
+      const size_t we = (size_t)nw * N * 2 * P->Kx * (P->prec == GW_3XTF32 ? 4 : 2);
+      for (int i = 0; i < (P->prec == GW_3XTF32 ? 4 : 6); ++i) {
+        uint8_t* pp;
+        ALLOC(pp, we);
+        P->d_Wpl.b[i] = pp;
+      }
+      const size_t vp = (size_t)(P->NK + (prob->head_wings ? 1 : 0)) * N;
+      for (auto& p : P->d_Vpc) ALLOC(p, vp * 2 * P->Kx);
+      ALLOC(P->d_Ve, vp / N);
+    }
+    if (!P->fp64) {
+      const size_t pe = (size_t)N * 2 * P->ldm * (P->prec == GW_3XTF32 ? 4 : 2);
+      ALLOC(P->d_Praw, (size_t)N * 2 * P->ldm);
+      P->n_bpl = P->prec == GW_3XBF16 ? 3 : 2;
+      ALLOC(P->d_absmax, 1);
+      ALLOC(P->d_hmax, std::max<size_t>(2 * (size_t)nw, P->NK + 1));
+      ALLOC(P->d_hrow, (size_t)nw * P->Kx);
+      ALLOC(P->d_hesc, (size_t)nw);
+      ALLOC(P->d_eB, 1);
+      ALLOC(P->d_escale, (size_t)nw);
+      for (int i = 0; i < P->n_bpl; ++i) {
+        uint8_t* pp;
+        ALLOC(pp, pe);
+        P->d_Pb[i] = pp;
+      }
+      ALLOC(P->d_wtab, (size_t)nw * P->ldm);
+      if (const char* e = std::getenv("GW_CHI0_SEG_ROWS")) P->seg_rows = std::max(32, std::atoi(e));
+      if (const char* e = std::getenv("GW_CHI0_COMPRESS_TOL")) P->compress_tol = std::max(0.0, std::atof(e));
+      if (nw <= 64) {
+        ALLOC(P->d_wG, (size_t)nw * nw * P->NK);
+        ALLOC(P->d_wU, (size_t)nw * nw * P->NK);
+        ALLOC(P->d_wlam, (size_t)nw * P->NK);
+        ALLOC(P->d_wn, (size_t)nw * P->NK);
+        ALLOC(P->d_wE, (size_t)nw * nw * P->NK);
+        ALLOC(P->d_wP, (size_t)nw * nw * P->NK);
+        ALLOC(P->d_werr, (size_t)nw * (nw + 1) * P->NK);
+        ALLOC(P->d_C, (size_t)nw * NN);
+      }
+    }
+    ALLOC(P->d_delta, P->ldm);
+    ALLOC(P->d_delta_f, P->ldm);
+    ALLOC(P->d_pq, P->ldm);
+    if (prob->head_wings == 2) {
+      ALLOC(P->d_pq3, 3 * (size_t)P->ldm);
+      ALLOC(P->d_A6, (size_t)nw * 6);
+      ALLOC(P->d_h3, (size_t)nw * 3 * N);
+      ALLOC(P->d_Y3, (size_t)nw * 3 * N);
+      ALLOC(P->d_G3, (size_t)nw * 3 * N);
+      ALLOC(P->d_m10, (size_t)nw * 10);
+      P->n_dirs = 128;
+      ALLOC(P->d_dirs, 4 * (size_t)P->n_dirs);
+    }
+    return GW_OK;
+  };
+#undef ALLOC
+  // first the sum of the buffers, taken as one allocation (a cudaMalloc and a cudaFree for each of ~45 buffers
+  // was a quarter of a small system's run); within a workspace limit that the sum passes, or where the one
+  // allocation fails, each buffer for itself
+  P->measuring = true;
+  s = allocate();
+  P->measuring = false;
+  if (s != GW_OK) return cleanup(s);
+  if (!P->ws_limit || P->arena_need <= P->ws_limit) {
+    ++g_alloc_count;
+    void* a = nullptr;
+    if (cudaMalloc(&a, P->arena_need) == cudaSuccess) {
+      P->arena = static_cast<uint8_t*>(a);
+      P->arena_size = P->arena_need;
+    } else {
+      cudaGetLastError();
+    }
   }
-  if (!P->fp64) {
-    const size_t pe = (size_t)N * 2 * P->ldm * (P->prec == GW_3XTF32 ? 4 : 2);
-    ALLOC(P->d_Praw, (size_t)N * 2 * P->ldm);
-    P->n_bpl = P->prec == GW_3XBF16 ? 3 : 2;
-    ALLOC(P->d_absmax, 1);
-    ALLOC(P->d_hmax, std::max<size_t>(2 * (size_t)nw, P->NK + 1));
-    ALLOC(P->d_hrow, (size_t)nw * P->Kx);
-    ALLOC(P->d_hesc, (size_t)nw);
-    ALLOC(P->d_eB, 1);
-    ALLOC(P->d_escale, (size_t)nw);
-    for (int i = 0; i < P->n_bpl; ++i) {
-      uint8_t* pp;
-      ALLOC(pp, pe);
-      P->d_Pb[i] = pp;
-    }
-    ALLOC(P->d_wtab, (size_t)nw * P->ldm);
-    if (const char* e = std::getenv("GW_CHI0_SEG_ROWS")) P->seg_rows = std::max(32, std::atoi(e));
-    if (const char* e = std::getenv("GW_CHI0_COMPRESS_TOL")) P->compress_tol = std::max(0.0, std::atof(e));
-    if (nw <= 64) {
-      ALLOC(P->d_wG, (size_t)nw * nw * P->NK);
-      ALLOC(P->d_wU, (size_t)nw * nw * P->NK);
-      ALLOC(P->d_wlam, (size_t)nw * P->NK);
-      ALLOC(P->d_wn, (size_t)nw * P->NK);
-      ALLOC(P->d_wE, (size_t)nw * nw * P->NK);
-      ALLOC(P->d_wP, (size_t)nw * nw * P->NK);
-      ALLOC(P->d_werr, (size_t)nw * (nw + 1) * P->NK);
-      ALLOC(P->d_C, (size_t)nw * NN);
-    }
-  }
-  ALLOC(P->d_delta, P->ldm);
-  ALLOC(P->d_delta_f, P->ldm);
-  ALLOC(P->d_pq, P->ldm);
+  if ((s = allocate()) != GW_OK) return cleanup(s);
   if (prob->head_wings == 2) {
-    ALLOC(P->d_pq3, 3 * (size_t)P->ldm);
-    ALLOC(P->d_A6, (size_t)nw * 6);
-    ALLOC(P->d_h3, (size_t)nw * 3 * N);
-    ALLOC(P->d_Y3, (size_t)nw * 3 * N);
-    ALLOC(P->d_G3, (size_t)nw * 3 * N);
-    ALLOC(P->d_m10, (size_t)nw * 10);
     // direction rule: 8 Gauss-Legendre nodes in cos(theta) x 16 equally spaced phi (half-step
     // offset), weights summing to one; symmetric under q^ -> -q^
     std::vector<double> u, wu, rule;
@@ -890,12 +935,9 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
         const double ph = 2.0 * M_PI * (j + 0.5) / 16.0, st = std::sqrt(1.0 - u[i] * u[i]);
         rule.insert(rule.end(), {st * std::cos(ph), st * std::sin(ph), u[i], wu[i] / 2.0 / 16.0});
       }
-    P->n_dirs = 128;
-    ALLOC(P->d_dirs, rule.size());
     if (cudaMemcpy(P->d_dirs, rule.data(), sizeof(double) * rule.size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return cleanup(fail(GW_ERR_CUDA, "direction rule upload failed"));
   }
-#undef ALLOC
   if (cudaEventCreate(&P->ev0) != cudaSuccess || cudaEventCreate(&P->ev1) != cudaSuccess)
     return cleanup(fail(GW_ERR_CUDA, "cudaEventCreate failed"));
   cudaStream_t st = P->st;
@@ -1018,7 +1060,9 @@ gw_status gw_plan_destroy(gw_plan P) {
   }
   if (P->st) cudaStreamSynchronize(P->st);
   else cudaDeviceSynchronize();
-  for (void* a : P->allocs) cudaFree(a);
+  for (void* a : P->allocs)
+    if (!in_arena(P, a)) cudaFree(a);
+  if (P->arena) cudaFree(P->arena);
   if (P->chi0plan) chi0_plan_free(P->chi0plan);
   if (P->ev0) cudaEventDestroy(P->ev0);
   if (P->ev1) cudaEventDestroy(P->ev1);
@@ -1612,10 +1656,8 @@ gw_status gw_qp(gw_plan P, int32_t sys, const gw_complex* sigma, const double* d
   if (!e_qp || !gap) return fail(GW_ERR_ARG, "e_qp and gap must not be NULL");
   cudaStream_t st = P->st;
   const int n = P->NK * P->nsig;
-  double* d_e;
-  int* d_c;
-  GW_TRY(dalloc(P, &d_e, n));
-  GW_TRY(dalloc(P, &d_c, n));
+  double* d_e = P->d_qp_e;
+  int* d_c = P->d_qp_c;
   const c128* sg = sigma ? reinterpret_cast<const c128*>(sigma) : P->d_sigma;
   launch_qp(P->NK, P->nsig, P->NBd, P->p.sigma_lo, P->nw, sg, dxv, P->p.eps, P->d_mu, P->d_freq, d_e, d_c, st);
   GW_TRY(check_launch(P, "gw_qp"));
@@ -1623,8 +1665,6 @@ gw_status gw_qp(gw_plan P, int32_t sys, const gw_complex* sigma, const double* d
   GW_CUDA(cudaMemcpyAsync(e_qp, d_e, n * sizeof(double), cudaMemcpyDeviceToHost, st));
   GW_CUDA(cudaMemcpyAsync(conv.data(), d_c, n * sizeof(int), cudaMemcpyDeviceToHost, st));
   GW_CUDA(cudaStreamSynchronize(st));
-  dfree_last(P);
-  dfree_last(P);
   int nc = 0;
   for (int i = 0; i < n; ++i) nc += conv[i];
   if (n_conv) *n_conv = nc;
@@ -2191,16 +2231,19 @@ gw_status gw_plan_n_sys(gw_plan P, int32_t* n_sys) {
 // Exchange self-energy (the bare-Coulomb part of Eq. GW_selfe_element, W = V + W^c):
 //   Sigma_x_n(k) = -(1/N_q) sum_q sum_{m occ} a^T V(q) a^*,  a = C_{nm}(k, k-q) = M_{nm}(k-q, q)
 // Rows a_r, r = ((kk * n_sigma) + n) * n_occ + m, as for Sigma_c but over the occupied bands;
-// U = A V(q) (FP64 GEMM on the FP64 path, FP32 on the split paths), S_r = Re U_r . conj(a_r).
+// U = A V(q) (FP64 GEMM on the FP64 path), S_r = Re U_r . conj(a_r); on the split paths one FP32 kernel over the
+// Hermitian triangle of V with the row dot in its epilogue (k_sigx_dot).
 // ---------------------------------------------------------------------------------------------
 namespace {
 
-__global__ void k_sigx_accum(int nkk, int kk0, int nsig, int nocc, const double* __restrict__ S, double scale,
+// sigx[k][n] += scale sum over the q of a group, the column blocks and the bands m of S[q][block][row]
+__global__ void k_sigx_accum(int nkk, int kk0, int nsig, int nocc, int parts, const double* __restrict__ S, double scale,
                              double* __restrict__ sigx) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nkk * nsig) return;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, n = nkk * nsig;
+  if (e >= n) return;
   double acc = 0.0;
-  for (int m = 0; m < nocc; ++m) acc += S[(long long)e * nocc + m];
+  for (int p = 0; p < parts; ++p)
+    for (int m = 0; m < nocc; ++m) acc += S[((long long)p * n + e) * nocc + m];
   sigx[(long long)kk0 * nsig + e] += scale * acc;
 }
 
@@ -2218,37 +2261,33 @@ gw_status gw_sigma_x(gw_plan P, int32_t sys, double* sigx) {
   const int N = P->N, nsig = P->nsig, nocc = P->nocc;
   const long long NN = (long long)N * N;
   const long long rows_max = (long long)P->sig_nkk * nsig * nocc;   // <= sig_rows
-  if (!P->d_Sx) {
-    GW_TRY(dalloc(P, &P->d_Sx, (size_t)rows_max));
-    if (!P->fp64) {
-      GW_TRY(dalloc(P, &P->d_Ux, (size_t)rows_max * P->Kx));
-      GW_TRY(dalloc(P, &P->d_Vx32, (size_t)NN));
-    }
-  }
+  // split path: as many q per product launch as the row buffer holds (8 at most: enough to fill the chip)
+  const int qg = P->fp64 ? 1 : (int)std::max<long long>(1, std::min<long long>(std::min(8, P->NK), P->sig_rows / rows_max));
+  const int nblk = P->fp64 ? 1 : sigx_blocks(N);
+  if (!P->d_Sx) GW_TRY(dalloc(P, &P->d_Sx, (size_t)rows_max * qg * nblk));
   const c128* evec = reinterpret_cast<const c128*>(P->p.evec);
   const c128* V = reinterpret_cast<const c128*>(P->p.V);
   GW_CUDA(cudaMemsetAsync(sigx, 0, sizeof(double) * P->NK * nsig, st));
-  for (int q = 0; q < P->NK; ++q) {
-    if (!P->fp64) launch_convert((long long)NN, V + q * NN, P->d_Vx32, st);
+  for (int q0 = 0; q0 < P->NK; q0 += qg) {
+    const int nq = std::min(qg, P->NK - q0);
     for (int kk0 = 0; kk0 < P->NK; kk0 += P->sig_nkk) {
       const int nkk = std::min(P->sig_nkk, P->NK - kk0);
       const int R = nkk * nsig * nocc;
       if (P->fp64) {
         c128* A = static_cast<c128*>(P->d_A);
         c128* U = static_cast<c128*>(P->d_U);
-        launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), evec, q, kk0, nkk,
+        launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), evec, q0, kk0, nkk,
                             MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, nocc, A, N, 1, st);
-        launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, V + q * NN, N, 0, OP_N, c128{0, 0}, U, N, 0, 1, st);
+        launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, V + q0 * NN, N, 0, OP_N, c128{0, 0}, U, N, 0, 1, st);
         launch_rowdot<double>(R, N, U, A, N, nullptr, P->d_Sx, 0, 1, st);
       } else {
         c64* A = static_cast<c64*>(P->d_A);
-        launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), P->d_evec32, q, kk0, nkk, MAP_K_IS_KK_MINUS_Q,
-                           P->p.sigma_lo, nsig, 0, nocc, A, P->Kx, 1, st);
-        launch_zgemm<float>(R, N, N, c64{1, 0}, A, P->Kx, 0, OP_N, P->d_Vx32, N, 0, OP_N, c64{0, 0}, P->d_Ux, P->Kx,
-                            0, 1, st);
-        launch_rowdot<float>(R, N, P->d_Ux, A, P->Kx, nullptr, P->d_Sx, 0, 1, st);
+        for (int j = 0; j < nq; ++j)
+          launch_mgen<float>(P->geom, static_cast<const c64*>(P->d_T1), P->d_evec32, q0 + j, kk0, nkk, MAP_K_IS_KK_MINUS_Q,
+                             P->p.sigma_lo, nsig, 0, nocc, A + (long long)j * R * P->Kx, P->Kx, 1, st);
+        launch_sigx_dot(R, N, P->Kx, A, V + q0 * NN, P->d_Sx, nq, st);
       }
-      ++g_launch_count, k_sigx_accum<<<(nkk * nsig + 127) / 128, 128, 0, st>>>(nkk, kk0, nsig, nocc, P->d_Sx,
+      ++g_launch_count, k_sigx_accum<<<(nkk * nsig + 127) / 128, 128, 0, st>>>(nkk, kk0, nsig, nocc, nq * nblk, P->d_Sx,
                                                                              -1.0 / P->NK, sigx);
     }
     GW_TRY(check_launch(P, "gw_sigma_x"));

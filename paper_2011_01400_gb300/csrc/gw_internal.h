@@ -92,6 +92,9 @@ void launch_row_dots(int rows, int cols, int K, double alpha, const c128* A, lon
 size_t inv_work_bytes(int N, int batch);
 gw_status launch_inv_minus_I(int N, c128* A, int batch, long long stride, void* work, int* status, cudaStream_t st,
                              std::string& err);
+// exchange products of nq consecutive q: S[q][sigx_blocks(N)][R] from the rows A [nq][R][ldA] and V [nq][N][N]
+int sigx_blocks(int N);
+void launch_sigx_dot(int R, int N, int ldA, const c64* A, const c128* V, double* S, int nq, cudaStream_t st);
 template <typename T> void launch_axpby_identity(int N, cplx<T>* A, long long s, int batch, T diag, cudaStream_t st);
 void launch_take_both(int N, const c128* C, long long s, int batch, float d, c64* X, c64* XH, cudaStream_t st);
 void launch_dev_identity(int N, const c64* T, long long total, unsigned* dev, cudaStream_t st);

@@ -165,6 +165,100 @@ __global__ void __launch_bounds__(256, 2) k_cgemm_nn(int m, int n, int k, c64 al
     }
 }
 
+// Exchange products: S[q][block][r] = Re sum_nu in block (sum_mu a_mu V_mu nu) conj(a_nu) with V(q) Hermitian, so
+// column block n0 sums mu from n0 on, those beyond its own 80 columns twice (V doubled as it is read: exact).
+// The tile of k_cgemm_nn with the row dot in the epilogue (FP64 sums) and the q of a group side by side; the
+// FP32 units bound it. 64 q of 2048 rows, N = 400: 5.7 -> 3.5 ms (whole products, FP32 rows of U written and
+// read again by a row-dot kernel, 130 blocks per launch).
+__global__ void __launch_bounds__(256, 2) k_sigx_dot(int R, int N, int ldA, const c64* __restrict__ A,
+                                                     const c128* __restrict__ V, double* __restrict__ S) {
+  __shared__ float2 As[2][CG_K][CG_AP];
+  __shared__ float2 Bs[2][CG_K][CG_T];
+  A += (long long)blockIdx.z * R * ldA;
+  V += (long long)blockIdx.z * N * N;
+  const int m0 = blockIdx.y * CG_T, n0 = blockIdx.x * CG_T;
+  const int t = threadIdx.x, tx = t % 16, ty = t / 16;
+  float2 ra[5], rb[5];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      const int e = t + 256 * c;
+      const int ar = m0 + e / CG_K, ak = k0 + e % CG_K;
+      ra[c] = (ar < R && ak < N) ? *reinterpret_cast<const float2*>(A + (long long)ar * ldA + ak) : make_float2(0.f, 0.f);
+      const int bk = k0 + e / CG_T, bc = n0 + e % CG_T;
+      rb[c] = make_float2(0.f, 0.f);
+      if (bk < N && bc < N) {
+        const c128 v = V[(long long)bk * N + bc];
+        const float f = bk >= n0 + CG_T ? 2.f : 1.f;
+        rb[c] = make_float2(f * (float)v.re, f * (float)v.im);
+      }
+    }
+  };
+  auto stash = [&](int buf) {
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      const int e = t + 256 * c;
+      As[buf][e % CG_K][e / CG_K] = ra[c];
+      Bs[buf][e / CG_T][e % CG_T] = rb[c];
+    }
+  };
+  float2 acc[5][5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int j = 0; j < 5; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  fetch(n0);
+  stash(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = n0; k0 < N; k0 += CG_K) {
+    const bool more = k0 + CG_K < N;
+    if (more) fetch(k0 + CG_K);
+#pragma unroll
+    for (int kk = 0; kk < CG_K; ++kk) {
+      float2 a[5], b[5];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) a[i] = As[buf][kk][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) b[j] = Bs[buf][kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+          acc[i][j].x = fmaf(a[i].x, b[j].x, acc[i][j].x);
+          acc[i][j].x = fmaf(-a[i].y, b[j].y, acc[i][j].x);
+          acc[i][j].y = fmaf(a[i].x, b[j].y, acc[i][j].y);
+          acc[i][j].y = fmaf(a[i].y, b[j].x, acc[i][j].y);
+        }
+    }
+    if (more) {
+      stash(buf ^ 1);
+      __syncthreads();
+      buf ^= 1;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const int gm = m0 + ty + 16 * i;
+    double s = 0.0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      const int gn = n0 + tx + 16 * j;
+      if (gm < R && gn < N) {
+        const float2 a = *reinterpret_cast<const float2*>(A + (long long)gm * ldA + gn);
+        s = fma((double)acc[i][j].x, (double)a.x, fma((double)acc[i][j].y, (double)a.y, s));
+      }
+    }
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (tx == 0 && gm < R) S[((long long)blockIdx.z * gridDim.x + blockIdx.x) * R + gm] = s;
+  }
+}
+int sigx_blocks(int N) { return (N + CG_T - 1) / CG_T; }
+void launch_sigx_dot(int R, int N, int ldA, const c64* A, const c128* V, double* S, int nq, cudaStream_t st) {
+  const dim3 grid(sigx_blocks(N), (R + CG_T - 1) / CG_T, nq);
+  ++::gw::g_launch_count, k_sigx_dot<<<grid, 256, 0, st>>>(R, N, ldA, A, V, S);
+}
+
 template <typename T>
 void launch_zgemm(int m, int n, int k, cplx<T> alpha, const cplx<T>* A, long long lda, long long sA, Op opA,
                   const cplx<T>* B, long long ldb, long long sB, Op opB, cplx<T> beta, cplx<T>* C, long long ldc,
