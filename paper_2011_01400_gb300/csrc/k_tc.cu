@@ -10,24 +10,29 @@
 // pieces are split before the launch (k_a_planes) and streamed by TMA like the B pieces.
 //
 // Accumulation. The tensor-core FP32 accumulator rounds every addition toward zero. hh goes to
-// accumulator D1, the correction products (2^-8 smaller) to D2; both are drained once per segment
-// into FP32 running sums held in registers by the epilogue warps (K = n_aux is short: at most 52
-// MMAs per item, a truncation bias ~1e-6 relative of S, far inside the Sigma_c tolerance).
+// accumulator D1, the correction products (2^-8 smaller) to D2; both are drained once per item into FP32
+// sums held in registers by the epilogue warps (a truncation bias ~1e-6 relative of S, far inside the
+// Sigma_c tolerance).
 //
-// Hermitian triangle: column block nb needs K = mu from its own block on; the block's own 64
-// ABFs form one segment (counted once), the rest a second one (counted twice, 2 Re).
+// Hermitian triangle: column block nb needs K = mu from its own block on, its own 64 ABFs counted once and
+// the rest twice (2 Re): the planes hold the diagonal blocks halved (exact), the sum is doubled.
 //
-// Work distribution: one CTA per SM, each walking the work items (row block, frequency, column
-// block; column block fastest, so that concurrent CTAs share their W^c tiles in L2); all
-// pipelines (barrier phases, TMEM buffers) run on across items.
+// Pairs of CTAs (clusters of two, cta_group::2): an item is 256 rows, 128 in each CTA, against the same 64
+// columns; CTA 0 holds B1, CTA 1 B2, and one MMA (M = 256, N = 128) reads both. Shared memory bounds the
+// kernel: a stage of 12 MMAs reads 8 KB of operands per MMA and CTA when a CTA works alone (96 KB, and 64 KB
+// written by TMA: 1280 of its 1540 clocks), 6 KB in a pair (72 KB and 48 KB: 940 of 1360). Measured, per q:
+// 216 k, N = 400, 32 frequencies 8.15 -> 7.53 ms; one k, N = 1600, TF32 4.90 -> 3.34 ms.
 //
-// Roles (384 threads):
-//   * warp 0 (TMA):   B1 / B2 pieces, 64 rows x 128 B each per stage, SWIZZLE_128B
-//   * warp 2 (TMA):   A pieces, 128 rows x 128 B each per stage; after each item's stages the
-//                     item's fp32 a tile (128 rows x BN complex) into the a-tile buffer for the
-//                     epilogue's row dot
-//   * warp 1:         one elected thread issues tcgen05.mma (M = 128, N = 128) into TMEM
-//   * warps 4-11:     epilogue (two warps per TMEM lane quadrant, 32 complex columns each)
+// Work distribution: one pair of CTAs per two SMs, each walking the work items (row block, frequency,
+// column block; column block fastest, so that concurrent pairs share their W^c tiles in L2); all pipelines
+// (barrier phases, TMEM buffers) run on across items.
+//
+// Roles (384 threads of each CTA):
+//   * warp 0 (TMA):   this CTA's half of the B pieces (64 rows x 128 B each) and its A pieces (128 rows x
+//                     128 B each) per stage, SWIZZLE_128B, completing on CTA 0's barrier
+//   * warp 2 (TMA):   the item's fp32 a tile (128 rows x BN complex) for the epilogue's row dot
+//   * warp 1:         in CTA 0 one elected thread issues tcgen05.mma into the TMEM of both CTAs
+//   * warps 4-11:     epilogue of this CTA's 128 rows (two warps per TMEM lane quadrant, 32 complex columns each)
 // All mbarrier waits are bounded; on expiry the kernel sets ST_TIMEOUT and unwinds.
 #include "gw_internal.h"
 #include "tc_ptx.cuh"
@@ -45,8 +50,8 @@ namespace {
 using namespace ptx;
 
 constexpr int BM = 128, BN = 64;                   // complex output tile
-constexpr int TILE = 128 * ROWB;                   // 16 KB: A piece (128 rows) or B piece ([B1; B2], 128 rows)
-constexpr int HALF = 64 * ROWB;                    // 8 KB: B1 or B2 part of a B piece
+constexpr int TILE = 128 * ROWB;                   // 16 KB: A piece (this CTA's 128 rows)
+constexpr int HALF = 64 * ROWB;                    // 8 KB: this CTA's half of a B piece (B1 in CTA 0, B2 in CTA 1)
 constexpr int RAW = 128 * ROWB;                    // 16 KB: one fp32 box (32 floats x 128 rows) of the a tile
 constexpr int RAW_BOXES = 2 * BN / 32;             // boxes of one BN-column a tile
 constexpr int NP = 2;                              // pieces per operand
@@ -55,8 +60,8 @@ constexpr int NTHREADS = 384;
 constexpr uint32_t D1_COL = 0, D2_COL = 256, DBUF = 128;
 
 template <bool TF32> struct Cfg {
-  static constexpr int STAGE = 2 * NP * TILE;      // B pieces then A pieces
-  static constexpr int STAGES = 2;
+  static constexpr int STAGE = NP * (HALF + TILE); // B pieces then A pieces: 48 KB
+  static constexpr int STAGES = 3;
   static constexpr int RS = TF32 ? 16 : 32;        // complex K entries per stage (128 B rows)
   static constexpr int BAR_OFF = STAGES * STAGE + RAW_BOXES * RAW;
   static constexpr int SMEM = BAR_OFF + 256 + 1024;
@@ -96,249 +101,223 @@ struct Maps {
   CUtensorMap a[2];   // A-side pieces (128 B x 128 rows per box)
 };
 
+// column blocks in the order 0, last, 1, last - 1, ...: a pair steps through the positions one by one, and a
+// short K range (a late block) between long ones leaves the epilogue the time it needs
 __device__ __forceinline__ void decode_item(const TcParams& p, int item, int& m0, int& n0, int& w) {
-  const int nb = item % p.nnb;
+  const int j = item % p.nnb, nb = (j & 1) ? p.nnb - 1 - j / 2 : j / 2;
   const int rest = item / p.nnb;
   w = rest % p.nw;
-  m0 = (rest / p.nw) * BM;
+  m0 = (rest / p.nw) * 2 * BM;
   n0 = nb * BN;
 }
 
-// the triangle's K range of column block n0 and its two segments
+// The triangle's K range of column block n0 starts at its own block; stage j of its `n` stages. The own
+// block, which holds the large diagonal of W^c, comes last: the accumulator truncates every addition, so the
+// small terms are summed before the large ones (with the own block first the error of S is 10x, N = 1600).
 template <int RS>
-__device__ __forceinline__ int first_stage(int n0) { return n0 / RS; }
+__device__ __forceinline__ int stages_of(int n0, int nst) { return nst - n0 / RS; }
 template <int RS>
-__device__ __forceinline__ bool is_seg_first(int i, int i0) { return i == i0 || i == i0 + BN / RS; }
-template <int RS>
-__device__ __forceinline__ bool is_seg_end(int i, int i0, int nst) { return i == nst - 1 || i == i0 + BN / RS - 1; }
+__device__ __forceinline__ int stage_at(int j, int n, int n0) {
+  const int own = min(BN / RS, n);
+  return n0 / RS + (j < n - own ? j + own : j - (n - own));
+}
 
 template <bool TF32>
-__global__ void __launch_bounds__(NTHREADS, 1) k_tc(const __grid_constant__ Maps maps, TcParams p) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) k_tc(const __grid_constant__ Maps maps, TcParams p) {
   using C = Cfg<TF32>;
   constexpr int STAGES = C::STAGES, STAGE = C::STAGE, RS = C::RS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* atile = smem + STAGES * STAGE;    // the item's fp32 a tile: RAW_BOXES boxes
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);
-  uint64_t* full_b = bars;                   // [STAGES]
-  uint64_t* full_a = bars + STAGES;          // [STAGES]
-  uint64_t* empty = bars + 2 * STAGES;       // [STAGES]
-  uint64_t* t1full = bars + 3 * STAGES;      // [2] D1 of a segment ready
-  uint64_t* t1empty = bars + 3 * STAGES + 2; // [2] D1 drained
-  uint64_t* t2full = bars + 3 * STAGES + 4;  // [2] D2 of a segment ready
-  uint64_t* t2empty = bars + 3 * STAGES + 6; // [2] D2 drained
-  uint64_t* done = bars + 3 * STAGES + 8;
-  uint64_t* tfull = bars + 3 * STAGES + 9;   // the a tile landed
-  uint64_t* tempty = bars + 3 * STAGES + 10; // the a tile read by the epilogue
-  uint32_t* tmem_base_p = reinterpret_cast<uint32_t*>(bars + 3 * STAGES + 11);
+  uint64_t* full = bars;                     // [STAGES] (CTA 0) both CTAs' operands landed
+  uint64_t* empty = bars + STAGES;           // [STAGES] the stage's MMAs are done
+  uint64_t* t1full = bars + 2 * STAGES;      // [2] D1 of an item ready
+  uint64_t* t1empty = bars + 2 * STAGES + 2; // [2] (CTA 0) D1 drained by both CTAs
+  uint64_t* t2full = bars + 2 * STAGES + 4;  // [2] D2 of an item ready
+  uint64_t* t2empty = bars + 2 * STAGES + 6; // [2] (CTA 0) D2 drained by both CTAs
+  uint64_t* tfull = bars + 2 * STAGES + 8;   // the a tile landed
+  uint64_t* tempty = bars + 2 * STAGES + 9;  // the a tile read by the epilogue
+  uint32_t* tmem_base_p = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 10);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full_b[s], 1);
-      mbar_init(&full_a[s], 1);
+      mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&t1full[b], 1);
-      mbar_init(&t1empty[b], 8);                // one per epilogue warp
+      mbar_init(&t1empty[b], 16);               // one per epilogue warp of the pair
       mbar_init(&t2full[b], 1);
-      mbar_init(&t2empty[b], 8);
+      mbar_init(&t2empty[b], 16);
     }
     mbar_init(tfull, 1);
     mbar_init(tempty, 8);
-    mbar_init(done, 1);
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(tmem_base_p, 512);
-    tmem_relinquish();
+    tmem_alloc_pair(tmem_base_p, 512);
+    tmem_relinquish_pair();
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();          // barriers of both CTAs are ready
   tc_fence_after();
+  const int rank = (int)cluster_rank();
+  const int pair = blockIdx.x / 2, npair = gridDim.x / 2;
   const uint32_t tmem = *tmem_base_p;
   const int nst = p.nstage;
 
   if (warp == 0) {
-    // ---------------- TMA producer: B1 / B2 pieces ----------------
+    // ---------------- TMA producer: this CTA's half of the B pieces and its A pieces ----------------
     if (lane == 0) {
       uint32_t gs = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+      for (int item = pair; item < p.n_items && ok; item += npair) {
         int m0, n0, w;
         decode_item(p, item, m0, n0, w);
-        const int yrow = w * p.Ncols + n0;
-        for (int i = first_stage<RS>(n0); i < nst; ++i, ++gs) {
+        const int yb = w * p.Ncols + n0, ya = m0 + rank * BM;
+        const int ns = stages_of<RS>(n0, nst);
+        for (int j = 0; j < ns; ++j, ++gs) {
           const int s = gs % STAGES;
           if (!mbar_wait(&empty[s], ((gs / STAGES) & 1) ^ 1, p.status)) { ok = false; break; }
           uint8_t* st = smem + s * STAGE;
-          mbar_arrive_expect_tx(&full_b[s], NP * TILE);
-          const int x = i * (ROWB / (TF32 ? 4 : 2));
+          const uint32_t bar = leader_addr(&full[s]);
+          if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * STAGE);
+          const int x = stage_at<RS>(j, ns, n0) * (ROWB / (TF32 ? 4 : 2));
 #pragma unroll
           for (int pc = 0; pc < NP; ++pc) {
-            tma_load_2d(st + pc * TILE, &maps.b[pc], &full_b[s], x, yrow);              // B1 rows 0..63
-            tma_load_2d(st + pc * TILE + HALF, &maps.b[NP + pc], &full_b[s], x, yrow);  // B2 rows 64..127
+            tma_load_2d_pair(st + pc * HALF, &maps.b[rank * NP + pc], bar, x, yb);
+            tma_load_2d_pair(st + NP * HALF + pc * TILE, &maps.a[pc], bar, x, ya);
           }
         }
       }
     }
   } else if (warp == 2) {
-    // ---------------- TMA producer: A pieces into the stages, then the item's a tile ----------------
+    // ---------------- TMA producer: the items' fp32 a tiles of the epilogue's row dot ----------------
     if (lane == 0) {
-      uint32_t gs = 0, gt = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+      uint32_t gt = 0;
+      for (int item = pair; item < p.n_items; item += npair, ++gt) {
         int m0, n0, w;
         decode_item(p, item, m0, n0, w);
-        for (int i = first_stage<RS>(n0); i < nst; ++i, ++gs) {
-          const int s = gs % STAGES;
-          if (!mbar_wait(&empty[s], ((gs / STAGES) & 1) ^ 1, p.status)) { ok = false; break; }
-          uint8_t* at = smem + s * STAGE + NP * TILE;
-          mbar_arrive_expect_tx(&full_a[s], NP * TILE);
-          const int x = i * (ROWB / (TF32 ? 4 : 2));
+        if (!mbar_wait(tempty, (gt & 1) ^ 1, p.status)) break;
+        mbar_arrive_expect_tx(tfull, RAW_BOXES * RAW);
 #pragma unroll
-          for (int pc = 0; pc < NP; ++pc) tma_load_2d(at + pc * TILE, &maps.a[pc], &full_a[s], x, m0);
-        }
-        if (ok) {
-          // the fp32 a tile of the epilogue's row dot (rows m0.., columns n0..n0+BN-1): issued after
-          // the item's stages, since it is read only at the item's end, once the previous item's
-          // epilogue has released the buffer
-          if (!mbar_wait(tempty, (gt & 1) ^ 1, p.status)) break;
-          mbar_arrive_expect_tx(tfull, RAW_BOXES * RAW);
-#pragma unroll
-          for (int c = 0; c < RAW_BOXES; ++c) tma_load_2d(atile + c * RAW, &maps.raw, tfull, 2 * n0 + 32 * c, m0);
-          ++gt;
-        }
+        for (int c = 0; c < RAW_BOXES; ++c)
+          tma_load_2d(atile + c * RAW, &maps.raw, tfull, 2 * n0 + 32 * c, m0 + rank * BM);
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    // ---------------- MMA issuer (CTA 0) ----------------
+    if (lane == 0 && rank == 0) {
       constexpr uint32_t fmt = TF32 ? 2u : 1u;
       const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)((2 * BN) >> 3) << 17) |
-                             ((uint32_t)(BM >> 4) << 24);
-      uint32_t gs = 0, gseg = 0;
+                             ((uint32_t)((2 * BM) >> 4) << 24);
+      int s = 0, b = 0;
+      uint32_t ph = 0, gitem = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+      for (int item = pair; item < p.n_items && ok; item += npair) {
         int m0, n0, w;
         decode_item(p, item, m0, n0, w);
-        const int i0 = first_stage<RS>(n0);
-        for (int i = i0; i < nst; ++i, ++gs) {
-          const int s = gs % STAGES;
-          const int b = gseg & 1;
-          const bool seg_first = is_seg_first<RS>(i, i0);
-          if (seg_first && gseg >= 2 && !mbar_wait(&t1empty[b], ((gseg >> 1) - 1) & 1, p.status)) {
-            ok = false;
-            break;
+        const int ns = stages_of<RS>(n0, nst);
+        for (int j = 0; j < ns; ++j) {
+          const bool first = j == 0;
+          if (first && gitem >= 2) {
+            const uint32_t par = ((gitem >> 1) - 1) & 1;
+            if (!mbar_wait_cluster(&t1empty[b], par, p.status) || !mbar_wait_cluster(&t2empty[b], par, p.status)) {
+              ok = false;
+              break;
+            }
           }
-          if (seg_first && gseg >= 2 && !mbar_wait(&t2empty[b], ((gseg >> 1) - 1) & 1, p.status)) {
-            ok = false;
-            break;
-          }
-          if (!mbar_wait(&full_b[s], (gs / STAGES) & 1, p.status)) { ok = false; break; }
-          if (!mbar_wait(&full_a[s], (gs / STAGES) & 1, p.status)) { ok = false; break; }
+          if (!mbar_wait_cluster(&full[s], ph, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t bbase = smem_u32(smem + s * STAGE);
-          const uint32_t abase = bbase + NP * TILE;
+          const uint64_t dB0 = sdesc(bbase), dB1 = sdesc(bbase + HALF);
+          const uint64_t dA0 = sdesc(bbase + NP * HALF), dA1 = sdesc(bbase + NP * HALF + TILE);
           const uint32_t d1 = tmem + D1_COL + b * DBUF;
           const uint32_t d2 = tmem + D2_COL + b * DBUF;
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint32_t ko = kk * 32;
-            const uint32_t acc = (seg_first && kk == 0) ? 0u : 1u;
-            const uint64_t A0 = sdesc(abase + ko), B0 = sdesc(bbase + ko);
-            const uint64_t A1 = sdesc(abase + TILE + ko), B1 = sdesc(bbase + TILE + ko);
-            mma<TF32>(d1, A0, B0, idesc, acc);
-            mma<TF32>(d2, A0, B1, idesc, acc);
-            mma<TF32>(d2, A1, B0, idesc, 1u);
+          for (int kk = 0; kk < 4; ++kk) {     // (a 32-byte K step adds 2 to the address field)
+            const uint32_t acc = (first && kk == 0) ? 0u : 1u;
+            mma_pair<TF32>(d1, dA0 + 2 * kk, dB0 + 2 * kk, idesc, acc);
+            mma_pair<TF32>(d2, dA0 + 2 * kk, dB1 + 2 * kk, idesc, acc);
+            mma_pair<TF32>(d2, dA1 + 2 * kk, dB0 + 2 * kk, idesc, 1u);
           }
-          mma_commit(&empty[s]);
-          if (is_seg_end<RS>(i, i0, nst)) {
-            mma_commit(&t1full[b]);
-            mma_commit(&t2full[b]);
-            ++gseg;
+          mma_commit_pair(&empty[s]);
+          if (j == ns - 1) {
+            mma_commit_pair(&t1full[b]);
+            mma_commit_pair(&t2full[b]);
+            ++gitem;
+            b ^= 1;
           }
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }
-      mma_commit(done);
-      mbar_wait(done, 0, p.status);
     }
   } else if (warp >= 4 && warp <= 11) {
-    // ---------------- epilogue: drain D1 and D2 per segment, row dot ----------------
+    // ---------------- epilogue: drain D1 and D2 per item, row dot ----------------
     const int quad = warp & 3;                 // TMEM lanes 32*quad .. 32*quad+31
     const int half = (warp - 4) >> 2;          // output columns half*32 .. half*32+31
     const int row = quad * 32 + lane;
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-    uint32_t gseg = 0, gt = 0;
-    bool ok = true;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+    uint32_t a1empty[2], a2empty[2];           // CTA 0's barriers
+    for (int b = 0; b < 2; ++b) {
+      a1empty[b] = leader_addr(&t1empty[b]);
+      a2empty[b] = leader_addr(&t2empty[b]);
+    }
+    uint32_t g = 0;
+    for (int item = pair; item < p.n_items; item += npair, ++g) {
       int m0, n0, w;
       decode_item(p, item, m0, n0, w);
-      const int m = m0 + row;
+      const int m = m0 + rank * BM + row;
       const int c0 = n0 + half * 32;
-      const int i0 = first_stage<RS>(n0);
-      bool tile_ready = false;
+      const int b = g & 1;
+      const uint32_t ph = (g >> 1) & 1;
       float sr[32], si[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) sr[j] = si[j] = 0.f;
-      for (int i = i0; i < nst; ++i) {
-        if (!is_seg_end<RS>(i, i0, nst)) continue;
-        const int b = gseg & 1;
-        const uint32_t ph = (gseg >> 1) & 1;
-        // every lane polls the barrier; reconverge before the warp-wide (.sync.aligned) TMEM loads
-        ok = __all_sync(0xffffffffu, mbar_wait(&t1full[b], ph, p.status));
-        if (!ok) break;
-        tc_fence_after();
-        drain_add(tmem + lane_off + D1_COL + b * DBUF + half * 32, sr, si);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&t1empty[b]);
-        ok = __all_sync(0xffffffffu, mbar_wait(&t2full[b], ph, p.status));
-        if (!ok) break;
-        tc_fence_after();
-        drain_add(tmem + lane_off + D2_COL + b * DBUF + half * 32, sr, si);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&t2empty[b]);
-        ++gseg;
-        const int nmax = p.Ncols - c0;
-        if (!tile_ready) {
-          ok = __all_sync(0xffffffffu, mbar_wait(tfull, gt & 1, p.status));
-          if (!ok) break;
-          tile_ready = true;
-        }
-        if (m < p.Mrows) {
-          // S_r += Re sum_nu U_{r nu} conj(a_{r nu}) over this thread's 32 columns, a from the a
-          // tile (complex column 32 half + j: box 2 half + j / 16, 16-B chunk (j % 16) / 2)
-          float acc = 0.f;
+      // every lane polls the barrier; reconverge before the warp-wide (.sync.aligned) TMEM loads
+      if (!__all_sync(0xffffffffu, mbar_wait(&t1full[b], ph, p.status))) break;
+      tc_fence_after();
+      drain_add(tmem + lane_off + D1_COL + b * DBUF + half * 32, sr, si);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(a1empty[b]);
+      if (!__all_sync(0xffffffffu, mbar_wait(&t2full[b], ph, p.status))) break;
+      tc_fence_after();
+      drain_add(tmem + lane_off + D2_COL + b * DBUF + half * 32, sr, si);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(a2empty[b]);
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull, g & 1, p.status))) break;
+      const int nmax = p.Ncols - c0;
+      if (m < p.Mrows) {
+        // S_r += 2 Re sum_nu U_{r nu} conj(a_{r nu}) over this thread's 32 columns (U with its own block
+        // halved), a from the a tile (complex column 32 half + j: box 2 half + j / 16, 16-B chunk (j % 16) / 2)
+        float acc = 0.f;
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const float4 a = *reinterpret_cast<const float4*>(atile + (2 * half + jj / 8) * RAW + swz(row, jj % 8));
-            if (2 * jj < nmax) acc = fmaf(sr[2 * jj], a.x, fmaf(si[2 * jj], a.y, acc));
-            if (2 * jj + 1 < nmax) acc = fmaf(sr[2 * jj + 1], a.z, fmaf(si[2 * jj + 1], a.w, acc));
-          }
-          // the diagonal block counts once, the strictly lower blocks twice (2 Re)
-          const float wgt = (i > i0 + (BN / RS) - 1) ? 2.f : 1.f;
-          atomicAdd(p.S + (long long)m * p.nw + w, wgt * acc);
+        for (int jj = 0; jj < 16; ++jj) {
+          const float4 a = *reinterpret_cast<const float4*>(atile + (2 * half + jj / 8) * RAW + swz(row, jj % 8));
+          if (2 * jj < nmax) acc = fmaf(sr[2 * jj], a.x, fmaf(si[2 * jj], a.y, acc));
+          if (2 * jj + 1 < nmax) acc = fmaf(sr[2 * jj + 1], a.z, fmaf(si[2 * jj + 1], a.w, acc));
         }
-#pragma unroll
-        for (int j = 0; j < 32; ++j) sr[j] = si[j] = 0.f;
-        if (i == nst - 1) {
-          // last segment of the item: release the a tile (generic reads before the TMA refill)
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty);
-          ++gt;
-        }
+        atomicAdd(p.S + (long long)m * p.nw + w, 2.f * acc);
       }
+      // release the a tile (generic reads before the TMA refill)
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty);
     }
   }
+  // neither CTA leaves while the other may read its operands, its TMEM or arrive on its barriers (the
+  // epilogues have waited for the last MMAs)
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, 512);
+  if (warp == 1) tmem_dealloc_pair(tmem, 512);
 }
 
 // chi0[w][i][j] = conj(chi0[w][j][i]) for i < j (the kernel writes lower tiles only)
@@ -385,8 +364,11 @@ __global__ void k_w_planes(int N, int nw, int Kpad, const c128* __restrict__ Wc,
     float v1[2] = {0.f, 0.f};
     if (mu < N) {
       const c128 w = Wc[row * N + mu];
-      v1[0] = (float)w.re;
-      v1[1] = conj ? -(float)w.im : (float)w.im;
+      // the diagonal blocks of BN columns count once, the rest of the triangle twice: halved here (exact),
+      // doubled with the sum
+      const float f = mu / BN == (int)(row % N) / BN ? 0.5f : 1.0f;
+      v1[0] = f * (float)w.re;
+      v1[1] = conj ? -f * (float)w.im : f * (float)w.im;
     }
     const float v2[2] = {-v1[1], v1[0]};
     const long long o = row * 2LL * Kpad + 2LL * mu;
@@ -468,7 +450,27 @@ template <bool TF32>
 gw_status launch_tc(const Maps& maps, const TcParams& p, cudaStream_t st, std::string& err) {
   const int smem = Cfg<TF32>::SMEM;
   cudaFuncSetAttribute(k_tc<TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  const int grid = std::min(p.n_items, num_sms());
+  // as many pairs of CTAs as run at once (an SM without a partner in its GPC stays out)
+  static std::atomic<int> resident{0};
+  int pairs = resident.load();
+  if (pairs == 0) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(num_sms() / 2 * 2);
+    cfg.blockDim = dim3(NTHREADS);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&pairs, k_tc<TF32>, &cfg) != cudaSuccess || pairs < 1) {
+      cudaGetLastError();
+      pairs = num_sms() / 2;
+    }
+    resident.store(pairs);
+  }
+  const int grid = 2 * std::min(p.n_items, pairs);
   ++::gw::g_launch_count, k_tc<TF32><<<grid, NTHREADS, smem, st>>>(maps, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -498,7 +500,7 @@ gw_status tc_sigma_run(const TcSigmaArgs& a, cudaStream_t st, std::string& err) 
     err = "tc_sigma: the A piece workspace is NULL";
     return GW_ERR_ARG;
   }
-  const int nmb = (a.R + BM - 1) / BM, nnb = (a.N + BN - 1) / BN;
+  const int nmb = (a.R + 2 * BM - 1) / (2 * BM), nnb = (a.N + BN - 1) / BN;
   const long long items = (long long)nmb * nnb * a.nw;
   if (items > 0x7fffffffLL) {
     err = "tc_sigma: too many work items";
