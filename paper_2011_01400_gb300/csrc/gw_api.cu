@@ -1435,7 +1435,7 @@ gw_status sigma_core(gw_plan_s* P, int q, const c128* Wc, c128* sig, bool conjW 
       for (int j = 0; j < nw; ++j) {
         launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, Wc + j * NN, N, 0, conjW ? OP_CONJ : OP_N,
                              c128{0, 0}, U, N, 0, 1, st);
-        launch_rowdot<double>(R, N, U, A, N, nullptr, P->d_S_d, j, nw, st);
+        launch_rowdot(R, N, U, A, N, P->d_S_d, j, nw, st);
       }
     } else {
       // rows a_r as an fp32 plane [R][Kx] (zero beyond n_aux), then the tensor-core contraction
@@ -1921,7 +1921,7 @@ gw_status sigma_core_sur(gw_plan_s* P, int q, const c128* Wc_c, const c128* U, c
                           MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, NBd, A, N, 1, st);
       for (int c = 0; c < nc; ++c) {
         launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, Wc_c + c * NN, N, 0, OP_N, c128{0, 0}, Ut, N, 0, 1, st);
-        launch_rowdot<double>(R, N, Ut, A, N, nullptr, S.d_Sc_d, c, nc, st);
+        launch_rowdot(R, N, Ut, A, N, S.d_Sc_d, c, nc, st);
       }
       c128* Pm = static_cast<c128*>(S.d_P);
       launch_zgemm<double>(R, k, N, c128{1, 0}, A, N, 0, OP_N, S.d_B, k, 0, OP_N, c128{0, 0}, Pm, k, 0, 1, st);
@@ -2279,7 +2279,7 @@ gw_status gw_sigma_x(gw_plan P, int32_t sys, double* sigx) {
         launch_mgen<double>(P->geom, static_cast<const c128*>(P->d_T1), evec, q0, kk0, nkk,
                             MAP_K_IS_KK_MINUS_Q, P->p.sigma_lo, nsig, 0, nocc, A, N, 1, st);
         launch_zgemm<double>(R, N, N, c128{1, 0}, A, N, 0, OP_N, V + q0 * NN, N, 0, OP_N, c128{0, 0}, U, N, 0, 1, st);
-        launch_rowdot<double>(R, N, U, A, N, nullptr, P->d_Sx, 0, 1, st);
+        launch_rowdot(R, N, U, A, N, P->d_Sx, 0, 1, st);
       } else {
         c64* A = static_cast<c64*>(P->d_A);
         for (int j = 0; j < nq; ++j)

@@ -128,9 +128,8 @@ void launch_midgap(int NK, int NBd, int nocc, const double* eps, double* mu, cud
 
 // k_sigma.cu
 // S[r][j] = Re sum_nu U[r][nu] conj(a[r][nu])
-template <typename T>
-void launch_rowdot(int R, int N, const cplx<T>* U, const cplx<T>* a, long long ld, float* S_f, double* S_d, int j,
-                   int nw, cudaStream_t st);
+void launch_rowdot(int R, int N, const c128* U, const c128* a, long long ld, double* S, int j, int nw,
+                   cudaStream_t st);
 // sigma[k][n][w] += pref * sum_m sum_j g_j S[(kk,n,m)][j] 2z/(z^2+w_j^2), z = i w + mu - eps_m(k-q),
 // for the target k = kk0 + kk of one chunk of rows r = ((kk*nsig)+n)*NBd + m.
 void launch_sigma_conv_chunk(int kk0, int nkk, int nsig, int NBd, const int* nk, int q, const double* eps,

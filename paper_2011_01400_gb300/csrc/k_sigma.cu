@@ -5,31 +5,22 @@
 namespace gw {
 
 // S[r][j] = Re sum_nu U[r][nu] conj(a[r][nu]) -- one warp per row.
-template <typename T>
-__global__ void k_rowdot(int R, int N, const cplx<T>* __restrict__ U, const cplx<T>* __restrict__ a, long long ld,
-                         float* S_f, double* S_d, int j, int nw) {
+__global__ void k_rowdot(int R, int N, const c128* __restrict__ U, const c128* __restrict__ a, long long ld, double* S,
+                         int j, int nw) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
   if (warp >= R) return;
-  const cplx<T>* u = U + (long long)warp * ld;
-  const cplx<T>* v = a + (long long)warp * ld;
+  const c128* u = U + (long long)warp * ld;
+  const c128* v = a + (long long)warp * ld;
   double s = 0;
-  for (int nu = lane; nu < N; nu += 32) s += (double)u[nu].re * v[nu].re + (double)u[nu].im * v[nu].im;
+  for (int nu = lane; nu < N; nu += 32) s += u[nu].re * v[nu].re + u[nu].im * v[nu].im;
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) {
-    if (S_d) S_d[(long long)warp * nw + j] = s;
-    if (S_f) S_f[(long long)warp * nw + j] = (float)s;
-  }
+  if (lane == 0) S[(long long)warp * nw + j] = s;
 }
-template <typename T>
-void launch_rowdot(int R, int N, const cplx<T>* U, const cplx<T>* a, long long ld, float* S_f, double* S_d, int j,
-                   int nw, cudaStream_t st) {
+void launch_rowdot(int R, int N, const c128* U, const c128* a, long long ld, double* S, int j, int nw,
+                   cudaStream_t st) {
   int blocks = (R * 32 + 255) / 256;
-  ++::gw::g_launch_count, k_rowdot<T><<<blocks, 256, 0, st>>>(R, N, U, a, ld, S_f, S_d, j, nw);
+  ++::gw::g_launch_count, k_rowdot<<<blocks, 256, 0, st>>>(R, N, U, a, ld, S, j, nw);
 }
-template void launch_rowdot<double>(int, int, const c128*, const c128*, long long, float*, double*, int, int,
-                                    cudaStream_t);
-template void launch_rowdot<float>(int, int, const c64*, const c64*, long long, float*, double*, int, int,
-                                   cudaStream_t);
 
 // sigma[k][n][w] += pref * sum_m sum_j g_j S[(kk,n,m)][j] 2 z / (z^2 + w_j^2),  z = i w + mu - eps_m(k - q)
 // Rows of S are r = ((kk * nsig) + n) * NBd + m for k = kk0 + kk. One block per (kk, n): thread
