@@ -1471,7 +1471,7 @@ gw_status sigma_core(gw_plan_s* P, int q, const c128* Wc, c128* sig, bool conjW 
 
 gw_status g0w0_sur(gw_plan_s* P, c128* sig);  // the surrogate pass, defined below
 
-// q-group buffers of gw_g0w0: chi0 (then W^c), eps~ (then eps~^-1 - 1), Cholesky scratch
+// q-group buffers of gw_g0w0: chi0 (then W^c), eps~ (then eps~^-1 - 1), scratch of the inverse
 gw_status ensure_groups(gw_plan_s* P) {
   if (P->g_chi0) return GW_OK;
   const long long slot = (long long)P->N * P->N * P->nw;
@@ -1686,11 +1686,7 @@ gw_status gw_qp(gw_plan P, int32_t sys, const gw_complex* sigma, const double* d
 
 // ---------------------------------------------------------------------------------------------
 // gw_qp_static: the QP solve of gw_qp with its device scratch (per-(k, n) energies and Newton
-// flags) in one fixed file-scope array instead of a cudaMalloc/cudaFree pair per call.
-// Callers that cannot allocate at that point use it: a process whose device memory is held by
-// a caching allocator (the pool is full, so a fresh cudaMalloc fails although the QP step
-// needs only a few hundred KB), and a serving loop that re-solves the QP equation after every
-// Sigma_c update and cannot take the device-wide synchronisation that cudaFree implies.
+// flags) in one fixed file-scope array instead of the plan's workspace. Neither call allocates.
 // The paper has no counterpart: it is a deployment variant of the QP step.
 // ---------------------------------------------------------------------------------------------
 #include <mutex>
