@@ -288,8 +288,8 @@ def timed_pass(gw, s, prec, torch, warm=1, qs=None, sigma=False):
 
 def fp64_gemm_peak(torch, n=4096, reps=5):
     """Measured FP64 rate of this GPU: the best of `reps` CUDA-event-timed cuBLAS DGEMMs
-    (torch.matmul, n^3, 2 n^3 flops) after one warm-up. It is the denominator of the FP64
-    Cholesky-inverse's roofline fraction (that kernel runs on the same FP64 units)."""
+    (torch.matmul, n^3, 2 n^3 flops) after one warm-up. It is what an inverse of eps~ on the
+    FP64 units would be bounded by (the library's runs its products on the tensor cores)."""
     a = torch.randn((n, n), dtype=torch.float64, device="cuda")
     b = torch.randn((n, n), dtype=torch.float64, device="cuda")
     c = torch.matmul(a, b)
@@ -748,7 +748,7 @@ def run_device(args, system, world, rank):
                                 dE_qp_argmax_k_band=[int(kn[0]), int(kn[1]) + s3.sigma_lo])
         line["fp64_pass"] = fp64_pass
     if world == 1 and not args.no_extras:
-        # the FP64 Cholesky-inverse of eps~: its share of the step and its FP64 rate against a
+        # the FP64 inverse of eps~: its operations per step, to set against a
         # measured FP64 GEMM (4 N^3 flops per (q, w) matrix: N^3 / 2 complex multiply-adds)
         peak64 = fp64_gemm_peak(torch)
         nq = q_computed(s)
