@@ -196,6 +196,7 @@ struct gw_plan_s {
   gw_problem p{};
   gw_precision prec;
   bool fp64;
+  bool conv64;                      // frequency convolution of Sigma_c in FP64
   cudaStream_t st = nullptr;
   int NK, N, NB, NBd, nocc, nunocc, nsig, nw, natoms;
   std::vector<int> basis_atom, aux_atom, R;
@@ -785,6 +786,8 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
       P->fweight[j] = 2.0 * prob->omega0 * w[j] / ((1.0 - x[j]) * (1.0 - x[j]));
     }
   }
+  // the FP32 convolution forms products up to w^4
+  P->conv64 = P->fp64 || *std::max_element(P->freq.begin(), P->freq.end()) > 1e9;
   const int N = P->N, nw = P->nw;
   const size_t NN = (size_t)N * N;
   gw_status s;
@@ -1463,7 +1466,7 @@ gw_status sigma_core(gw_plan_s* P, int q, const c128* Wc, c128* sig, bool conjW 
       }
     }
     launch_sigma_conv_chunk(kk0, nkk, nsig, NBd, P->p.nk, q, P->p.eps, P->d_mu, P->d_S_f, P->d_S_d, P->d_freq,
-                            P->d_fw, nw, pref, sig, P->fp64, st, ktab);
+                            P->d_fw, nw, pref, sig, P->conv64, st, ktab);
     GW_TRY(check_launch(P, "Sigma_c"));
   }
   return GW_OK;
@@ -1950,7 +1953,7 @@ gw_status sigma_core_sur(gw_plan_s* P, int q, const c128* Wc_c, const c128* U, c
       launch_sur_assemble<float>(R, nc, nw, k, S.d_jmap, S.d_Sc, Pm, coef, nf, Lmat, P->d_S_f, st);
     }
     launch_sigma_conv_chunk(kk0, nkk, nsig, NBd, P->p.nk, q, P->p.eps, P->d_mu, P->d_S_f, P->d_S_d, P->d_freq,
-                            P->d_fw, nw, pref, sig, P->fp64, st);
+                            P->d_fw, nw, pref, sig, P->conv64, st);
     GW_TRY(check_launch(P, "Sigma_c (surrogate)"));
   }
   return GW_OK;

@@ -131,7 +131,8 @@ void launch_midgap(int NK, int NBd, int nocc, const double* eps, double* mu, cud
 void launch_rowdot(int R, int N, const c128* U, const c128* a, long long ld, double* S, int j, int nw,
                    cudaStream_t st);
 // sigma[k][n][w] += pref * sum_m sum_j g_j S[(kk,n,m)][j] 2z/(z^2+w_j^2), z = i w + mu - eps_m(k-q),
-// for the target k = kk0 + kk of one chunk of rows r = ((kk*nsig)+n)*NBd + m.
+// for the target k = kk0 + kk of one chunk of rows r = ((kk*nsig)+n)*NBd + m. S from S_d, or from S_f where that
+// is NULL; fp64: the arithmetic (FP32 overflows beyond w = 1e9).
 void launch_sigma_conv_chunk(int kk0, int nkk, int nsig, int NBd, const int* nk, int q, const double* eps,
                              const double* mu, const float* S_f, const double* S_d, const double* freq,
                              const double* gw, int nw, double pref, c128* sigma, bool fp64, cudaStream_t st,
