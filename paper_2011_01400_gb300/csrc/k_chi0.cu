@@ -68,6 +68,14 @@ constexpr int TP_F16 = 1, TP_TF32 = 1;   // weight rows per work item (measured:
 
 enum { K_F16 = 0, K_BF16 = 1, K_TF32 = 2 };
 
+// F16: exponent s of the scale 2^s that takes a largest element m into [2^13, 2^14), at most 126 so that the
+// scale is a finite float (an m below 2^-113 stays below 2^13: its two pieces still hold 2^-36 absolutely)
+__device__ __forceinline__ int f16_scale(float m) {
+  int e = 0;
+  if (m > 0.f) frexpf(m, &e);              // m = f 2^e, f in [0.5, 1)
+  return min(14 - e, 126);
+}
+
 // Shared memory: a ring of SB B stages (TMA runs up to SB - 1 stages ahead of the MMAs, which
 // covers the L2 / HBM latency), SA buffers of split A pieces (written by the transform just in
 // time), and the raw-row ring of RING slots with their weights.
@@ -589,11 +597,9 @@ __global__ void k_b_pieces(long long n, const float* __restrict__ raw, const uns
                            void* p0, void* p1, void* p2, int* eB_out) {
   float s = 1.0f;
   if (KIND == K_F16) {
-    int e = 0;
-    const float m = __uint_as_float(*absmax);
-    if (m > 0.f) frexpf(m, &e);             // m = f 2^e, f in [0.5, 1)
-    s = ldexpf(1.0f, 14 - e);                // largest |x s| in [2^13, 2^14)
-    if (blockIdx.x == 0 && threadIdx.x == 0) *eB_out = 14 - e;
+    const int e = f16_scale(__uint_as_float(*absmax));   // largest |x s| in [2^13, 2^14)
+    s = ldexpf(1.0f, e);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *eB_out = e;
   }
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const float2 y = reinterpret_cast<const float2*>(raw)[e];
@@ -642,10 +648,7 @@ __global__ void k_wscale(int Kpad, int T, float* __restrict__ wtab, const unsign
     if (threadIdx.x == 0) red[0] = m;
   }
   __syncthreads();
-  const float bound = red[0] * __uint_as_float(*absmax);   // >= every |v_t(r) M^mu_r|
-  int e = 0;
-  if (bound > 0.f) frexpf(bound, &e);
-  const int eA = 14 - e;
+  const int eA = f16_scale(red[0] * __uint_as_float(*absmax));   // (the product is >= every |v_t(r) M^mu_r|)
   const float s = ldexpf(1.0f, eA);
   for (int r = threadIdx.x; r < Kpad; r += blockDim.x) w[r] *= s;
   if (threadIdx.x == 0) escale[t] = ldexp(scale, -(eA + *eB));
@@ -926,11 +929,9 @@ __global__ void k_h_pieces(int N, int Kpad, const cplx<T>* __restrict__ H, const
   const int b = blockIdx.y;
   float s = 1.0f;
   if constexpr (KIND == K_F16) {
-    int e = 0;
-    const float m = __uint_as_float(amax[b]);
-    if (m > 0.f) frexpf(m, &e);
-    s = ldexpf(1.0f, 14 - e);
-    if (blockIdx.x == 0 && threadIdx.x == 0) eB[b] = 14 - e;
+    const int e = f16_scale(__uint_as_float(amax[b]));
+    s = ldexpf(1.0f, e);
+    if (blockIdx.x == 0 && threadIdx.x == 0) eB[b] = e;
   }
   const long long total = (long long)N * Kpad;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -973,12 +974,7 @@ __global__ void k_round_max(long long n, const c128* __restrict__ in, c64* __res
 __global__ void k_herm_scales(int Kpad, const unsigned* __restrict__ amaxA, const int* __restrict__ eB, int f16,
                               double alpha, float* __restrict__ wrow, double* __restrict__ escale) {
   const int t = blockIdx.x;
-  int eA = 0;
-  if (f16) {
-    const float m = __uint_as_float(amaxA[t]);
-    if (m > 0.f) frexpf(m, &eA);
-    eA = 14 - eA;
-  }
+  const int eA = f16 ? f16_scale(__uint_as_float(amaxA[t])) : 0;
   for (int k = threadIdx.x; k < Kpad; k += blockDim.x) wrow[(long long)t * Kpad + k] = ldexpf(1.0f, eA);
   if (threadIdx.x == 0) escale[t] = ldexp(alpha, -(eA + (f16 ? *eB : 0)));
 }
