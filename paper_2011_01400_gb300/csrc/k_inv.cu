@@ -16,9 +16,15 @@
 // of two to 55-bit integers and cut into 7 balanced base-256 digits, exact in FP16. Products of
 // digits d1, d2 are summed in FP32 accumulators by order d1 + d2 = 0..6 (28 of the 49 pairs): at
 // most 7 pairs x 64 terms x 2^14 < 2^23, so every sum is an exact integer. The seven sums are put
-// together in 64-bit integers and rounded to FP64 once. What is dropped (orders above 6) is below
-// 2^-51 of the largest product of the two rows, the size of the rounding of an FP64 dot product of
-// 64 terms.
+// together in 64-bit integers and rounded to FP64 once. The dropped orders, above 6, are typically 2^-51
+// of the product of the two rows' largest elements (digits of random sign; 2^-45 if every digit were -128),
+// the size of the rounding of an FP64 dot product of 64 terms of that size.
+//
+// Scaling: an element 2^m below its row's largest is known to m bits less, so the error of a matrix D A D,
+// D diagonal, would grow with the spread of D (which it does not in FP64 elimination): 5e-13 at a spread
+// of 1e4, 4e-11 at 1e6. Rows and columns are therefore scaled by powers of two of the diagonal first, which is
+// exact and leaves 4e-16 at every spread (N = 200, against 5e-16 for FP64 Cholesky). eps~ with its
+// diagonal in [1, 4), the usual one, is not touched: the pass costs the two launches.
 //
 // Why: the chip does ~2 FP64 FMA per clock and SM (1.1 TFLOP/s by cuBLAS DGEMM) and the 4 N^3 flops
 // of an inverse bound the screening by that; 28 FP16 products of the tensor cores are ~25 times
@@ -123,9 +129,9 @@ __device__ __forceinline__ double pow2(int ex) {
 __host__ __device__ __forceinline__ int padded(int N) { return (N + TM - 1) / TM * TM; }
 
 // per-matrix workspace: digits of Y as right rows (yb) and as stacked left rows (ya), of W as left
-// rows, of W^H as right rows, and the rows' exponents
+// rows, of W^H as right rows, the rows' exponents, and the scales of A
 struct InvLayout {
-  long long yb, ya, w, r, ey, ew, er;   // byte offsets of the arrays over the batch
+  long long yb, ya, w, r, ey, ew, er, sc;   // byte offsets of the arrays over the batch
   long long bytes;
 };
 InvLayout inv_layout(int N, int batch) {
@@ -138,7 +144,8 @@ InvLayout inv_layout(int N, int batch) {
   l.ey = l.r + (long long)batch * ND * R_PLANE;
   l.ew = l.ey + (long long)batch * Nr * 4;
   l.er = l.ew + (long long)batch * PB * 4;
-  l.bytes = l.er + (long long)batch * PB * 4;
+  l.sc = l.er + (long long)batch * PB * 4;
+  l.bytes = l.sc + (long long)batch * N * 4;
   return l;
 }
 
@@ -148,6 +155,43 @@ __device__ __forceinline__ int row_field(const double (&x)[8], int& e) {
   for (int o = 1; o < 8; o <<= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
   e = f == 2047 ? E_BAD : (f == 0 ? 0 : f - 1022);
   return f;
+}
+
+// ---- scaling: A_ij <- 2^(s_i + s_j) A_ij with s_i taking the diagonal to [1, 4) ------------------
+
+__global__ void k_inv_exps(int N, const c128* __restrict__ Aall, long long stride, int* __restrict__ sc) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const double d = Aall[blockIdx.y * stride + (long long)i * (N + 1)].re;
+  sc[(long long)blockIdx.y * N + i] = d > 0.0 && isfinite(d) ? -(ilogb(d) >> 1) : 0;
+}
+
+// the scales of the 32 memory rows from j0 and of the 32 columns from i0; false if all are zero
+__device__ __forceinline__ bool tile_scales(int N, const int* __restrict__ sc, int j0, int i0, int (&se)[64]) {
+  const int t = threadIdx.y * 32 + threadIdx.x, r = t < 32 ? j0 + t : i0 + t - 32;
+  int s = 0;
+  if (t < 64) {
+    s = r < N ? sc[r] : 0;
+    se[t] = s;
+  }
+  return __syncthreads_or(s) != 0;
+}
+
+// The kept triangle of A; tiles whose scales are all zero are not touched
+__global__ void k_inv_scale(int N, c128* __restrict__ Aall, long long stride, const int* __restrict__ sc) {
+  __shared__ int se[64];
+  if (blockIdx.x < blockIdx.y) return;
+  c128* A = Aall + blockIdx.z * stride;
+  const int j0 = blockIdx.y * 32, i0 = blockIdx.x * 32;
+  if (!tile_scales(N, sc + (long long)blockIdx.z * N, j0, i0, se)) return;
+  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    const int j = j0 + r, i = i0 + threadIdx.x;
+    if (j < N && i < N && i >= j) {
+      const double fj = pow2(se[r]), fi = pow2(se[32 + threadIdx.x]);   // (one after the other: no overflow)
+      c128& a = A[(long long)j * N + i];
+      a = c128{a.re * fj * fi, a.im * fj * fi};
+    }
+  }
 }
 
 // ---- pivot block: W = L^{-1}, B_PP <- -W^H W ----------------------------------------------------
@@ -619,16 +663,20 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_inv_update(const __grid_cons
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// A := -B - I in full from the kept triangle
-__global__ void k_inv_finish(int N, c128* __restrict__ Aall, long long stride) {
+// A := -B - I in full from the kept triangle, the scales of A undone
+__global__ void k_inv_finish(int N, c128* __restrict__ Aall, long long stride, const int* __restrict__ sc) {
   __shared__ c128 tt[32][33];
+  __shared__ int se[64];
   if (blockIdx.x < blockIdx.y) return;
   c128* A = Aall + blockIdx.z * stride;
   const int j0 = blockIdx.y * 32, i0 = blockIdx.x * 32;     // memory rows j, columns i >= j
+  tile_scales(N, sc + (long long)blockIdx.z * N, j0, i0, se);
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int j = j0 + r, i = i0 + threadIdx.x;
     if (j < N && i < N && i >= j) {
-      const c128 v = A[(long long)j * N + i];
+      c128 v = A[(long long)j * N + i];
+      const double fj = pow2(se[r]), fi = pow2(se[32 + threadIdx.x]);
+      v = c128{v.re * fj * fi, v.im * fj * fi};
       const c128 o = i == j ? c128{-v.re - 1.0, 0.0} : c128{-v.re, -v.im};
       A[(long long)j * N + i] = o;
       tt[r][threadIdx.x] = o;
@@ -664,6 +712,10 @@ gw_status launch_inv_minus_I(int N, c128* A, int batch, long long stride, void* 
     return GW_ERR_CUDA;
   cudaFuncSetAttribute(k_inv_y, cudaFuncAttributeMaxDynamicSharedMemorySize, Y_SMEM);
   cudaFuncSetAttribute(k_inv_update, cudaFuncAttributeMaxDynamicSharedMemorySize, UPD_SMEM);
+  int* sc = reinterpret_cast<int*>(w + l.sc);
+  const int nt = (N + 31) / 32;
+  ++g_launch_count, k_inv_exps<<<dim3((N + 127) / 128, batch), 128, 0, st>>>(N, A, stride, sc);
+  ++g_launch_count, k_inv_scale<<<dim3(nt, nt, batch), dim3(32, 8), 0, st>>>(N, A, stride, sc);
   for (int p = 0; p < N; p += PB) {
     ++g_launch_count, k_inv_pivot<<<batch, PIV_THREADS, 0, st>>>(N, p, A, stride, w + l.w, w + l.r, eW, eR, status);
     if (N <= PB) break;
@@ -672,8 +724,7 @@ gw_status launch_inv_minus_I(int N, c128* A, int batch, long long stride, void* 
     ++g_launch_count, k_inv_update<<<nblk * batch, UPD_THREADS, UPD_SMEM, st>>>(maps, N, Nr, p, batch, A, stride, eY, eR,
                                                                                status);
   }
-  const int nt = (N + 31) / 32;
-  ++g_launch_count, k_inv_finish<<<dim3(nt, nt, batch), dim3(32, 8), 0, st>>>(N, A, stride);
+  ++g_launch_count, k_inv_finish<<<dim3(nt, nt, batch), dim3(32, 8), 0, st>>>(N, A, stride, sc);
   return GW_OK;
 }
 
