@@ -1,5 +1,6 @@
-"""The inverse of eps~ = 1 + D K D with the auxiliary functions' scales D spread over several powers of ten: the
-error of elimination does not depend on D. With V = 1 the screened interaction is the inverse itself."""
+"""Accuracy of the FP64 inverse of eps~, measured against LAPACK's own error: evenly scaled matrices up to
+kappa = 5e8, and eps~ = 1 + D K D with the auxiliary functions' scales D spread over several powers of ten (the error
+of elimination does not depend on D). With V = 1 the screened interaction is the inverse itself."""
 import numpy as np
 import pytest
 
@@ -9,11 +10,10 @@ pytestmark = pytest.mark.gpu
 
 
 def refined_inverse(e):
-    """Inverse to well below 2^-53: LAPACK's and Newton steps in extended precision."""
-    x, el, one = np.linalg.inv(e).astype(np.clongdouble), e.astype(np.clongdouble), np.eye(len(e))
-    for _ in range(3):
-        x = x + x @ (one - el @ x)
-    return x
+    """LAPACK's inverse and one Newton step with its residual in extended precision: error (u kappa)^2 + u (u kappa)."""
+    x = np.linalg.inv(e)
+    res = (np.eye(len(e)) - e.astype(np.clongdouble) @ x.astype(np.clongdouble)).astype(complex)
+    return x.astype(np.clongdouble) + x @ res
 
 
 def errors(e, x):
@@ -40,6 +40,15 @@ def system(n_aux, spread):
     return s
 
 
+def even_system(n_aux, strength):
+    """K of 54 pair rows: eps~ has eigenvalues 1 and up to strength^2 times as many tenths."""
+    cfg = dict(nk=(2, 1, 1), n_atoms=1, nb_per_atom=12, naux_per_atom=n_aux, n_bands=12, n_occ=3, n_freq=3,
+               sigma=(1, 4), omega_cell=100.0)
+    s = make_system(cfg, seed=n_aux, head_wings=0, c_scale=strength * 0.206 / np.sqrt(n_aux))
+    s.V[:] = np.eye(n_aux)
+    return s
+
+
 @pytest.mark.parametrize("n_aux", [24, 64, 129, 200])
 @pytest.mark.parametrize("spread", [1e2, 1e4, 1e6])
 def test_spread_rows(n_aux, spread):
@@ -50,6 +59,29 @@ def test_spread_rows(n_aux, spread):
     plan = gw.gw_plan_create(pb.prob)
     try:
         chi = torch.empty((2, n_aux, n_aux), dtype=torch.complex128, device="cuda")
+        w = torch.empty_like(chi)
+        gw.gw_chi0(plan, 0, 1, chi)
+        gw.gw_screen(plan, 0, 1, w)
+        chi, w = chi.cpu().numpy(), w.cpu().numpy()
+    finally:
+        gw.gw_plan_destroy(plan)
+    for c, x in zip(chi, w):
+        err, bound = errors(np.eye(n_aux) - c, x)
+        assert err <= bound
+
+
+@pytest.mark.parametrize("n_aux", [33, 65, 129, 200])
+@pytest.mark.parametrize("strength", [1.0, 300.0, 2e4])
+def test_even_rows(n_aux, strength):
+    """The bound is 2 to 200 times the kernel's error, which is 200 times larger without the last order of digit
+    products: from n_aux = 65 on every case fails then."""
+    torch = pytest.importorskip("torch")
+    from paper_2011_01400_gb300 import gw
+    s = even_system(n_aux, strength)
+    pb = gw.Problem(s, "fp64")
+    plan = gw.gw_plan_create(pb.prob)
+    try:
+        chi = torch.empty((3, n_aux, n_aux), dtype=torch.complex128, device="cuda")
         w = torch.empty_like(chi)
         gw.gw_chi0(plan, 0, 1, chi)
         gw.gw_screen(plan, 0, 1, w)
