@@ -34,7 +34,9 @@
  *   - Environment (read at gw_plan_create, all precisions):
  *     GW_WORKSPACE_LIMIT    bytes of device memory one plan may allocate for its workspace
  *                           (default: no limit). An allocation that would pass it fails with
- *                           GW_ERR_NOMEM before cudaMalloc is called.
+ *                           GW_ERR_NOMEM before cudaMalloc is called;
+ *     GW_INJECT_TIMEOUT     for tests of a caller's error handling: the named products (eps, sigma)
+ *                           of a split precision report an expired wait although they ran.
  */
 #ifndef GW_H
 #define GW_H
@@ -163,7 +165,7 @@ gw_status gw_chi0(gw_plan plan, int32_t sys, int32_t q, gw_complex* chi0_out);
  * with the head and wings of Eq. dielectric_func_gamma (insulator: f' term dropped).
  * Uses the chi0 of the last gw_chi0 call, which must be for the same q (else GW_ERR_STATE).
  * wc_out: device [n_freq][n_aux][n_aux] or NULL. eps~ is factorised and inverted in FP64.
- * Errors: GW_ERR_STATE, GW_ERR_NOT_PD, GW_ERR_CUDA. */
+ * Errors: GW_ERR_STATE, GW_ERR_NOT_PD, GW_ERR_CUDA, GW_ERR_TIMEOUT. */
 gw_status gw_screen(gw_plan plan, int32_t sys, int32_t q, gw_complex* wc_out);
 
 /* Adds the q term of Eq. (GW_selfe_element) with W^c in place of W:
@@ -172,7 +174,9 @@ gw_status gw_screen(gw_plan plan, int32_t sys, int32_t q, gw_complex* wc_out);
  *   z = i w + mu - eps_m(k-q), n in [sigma_lo, sigma_hi), m over all bands.
  * Uses the W^c of the last gw_screen call, which must be for the same q (else GW_ERR_STATE).
  * sigma_acc: device [N_k][sigma_hi-sigma_lo][n_freq], accumulated into (caller zeroes it),
- *            or NULL to accumulate into the plan's own buffer (zeroed at plan creation). */
+ *            or NULL to accumulate into the plan's own buffer (zeroed at plan creation).
+ * Does not wait for the device: a contraction that stalled is reported (GW_ERR_TIMEOUT) by the plan's next
+ * call that does, gw_chi0, gw_screen, gw_g0w0, gw_g0w0_qset, gw_g0w0_batch, gw_qp or gw_qp_static. */
 gw_status gw_sigma(gw_plan plan, int32_t sys, int32_t q, gw_complex* sigma_acc);
 
 /* The q term of Sigma_c (as gw_sigma) with a caller-supplied W^c(q) (device [n_freq][n_aux][n_aux],
@@ -180,7 +184,7 @@ gw_status gw_sigma(gw_plan plan, int32_t sys, int32_t q, gw_complex* sigma_acc);
  * (gw_problem.k_offset = k0), with the W^c of an unshifted plan of the same system, the sum over
  * q gives Sigma_c at the off-mesh points k0 + mesh (point 0 is k0 itself): band energies along
  * lines through the Brillouin zone. sigma_acc: device [N_k][n_sigma][n_freq] (rows outside the
- * k range untouched) or NULL for the plan's own accumulator.
+ * k range untouched) or NULL for the plan's own accumulator. A stalled contraction is reported as for gw_sigma.
  * Errors: GW_ERR_ARG (q, k range, NULL wc), GW_ERR_CUDA. */
 gw_status gw_sigma_ext(gw_plan plan, int32_t sys, int32_t q, const gw_complex* wc, int32_t k_lo, int32_t k_hi,
                        gw_complex* sigma_acc);
@@ -230,7 +234,8 @@ gw_status gw_plan_n_sys(gw_plan plan, int32_t* n_sys);
  * dxv:    device [N_k][n_sigma] (Sigma_x - v_xc) or NULL for zero.
  * e_qp:   host [N_k][n_sigma] output.
  * gap:    host scalar output, min_k E_LUMO - max_k E_HOMO when both are in the window, else NaN.
- * n_conv: host scalar output (may be NULL): number of (k, n) whose Newton iteration converged. */
+ * n_conv: host scalar output (may be NULL): number of (k, n) whose Newton iteration converged.
+ * Errors: GW_ERR_ARG, GW_ERR_CUDA, and GW_ERR_TIMEOUT of an earlier gw_sigma / gw_sigma_ext on this plan. */
 gw_status gw_qp(gw_plan plan, int32_t sys, const gw_complex* sigma, const double* dxv,
                 double* e_qp, double* gap, int32_t* n_conv);
 

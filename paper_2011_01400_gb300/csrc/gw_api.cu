@@ -213,6 +213,7 @@ struct gw_plan_s {
   std::vector<size_t> alloc_bytes;  // size of each entry of allocs
   size_t ws_bytes = 0;              // sum of alloc_bytes
   size_t ws_limit = 0;              // GW_WORKSPACE_LIMIT (bytes; 0 = no limit)
+  std::string inject;               // GW_INJECT_TIMEOUT
   int dev = -1;                     // CUDA device that was current at gw_plan_create
   bool trs = false;                 // time-reversal symmetric inputs (gw_problem.time_reversal)
   // time reversal without a q -> 0 direction: Sigma_c(-k) = Sigma_c(k), so gw_g0w0 computes the
@@ -409,6 +410,13 @@ gw_status check_launch(gw_plan_s* P, const char* where) {
   return GW_OK;
 }
 
+// GW_INJECT_TIMEOUT: the stage's products flag an expired wait (the word is all that a stalled pipeline leaves)
+void inject_timeout(gw_plan_s* P, const char* stage) {
+  if (P->inject == stage) cudaMemsetAsync(P->d_status, ST_TIMEOUT, 1, P->st);
+}
+
+// The status word is zeroed once, when the plan is created: a flag of a call that does not synchronise (gw_sigma,
+// gw_sigma_ext) stays until a call that does reads it here. What is read as an error ends the use of the plan.
 gw_status read_status(gw_plan_s* P, const char* where) {
   int st = 0;
   cudaError_t e = cudaMemcpyAsync(&st, P->d_status, sizeof(int), cudaMemcpyDeviceToHost, P->st);
@@ -726,6 +734,7 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
     const double lim = std::atof(v);
     if (lim > 0) P->ws_limit = (size_t)lim;
   }
+  if (const char* v = std::getenv("GW_INJECT_TIMEOUT")) P->inject = v;
   auto cleanup = [&](gw_status s) {
     std::string msg = g_last_error;
     gw_plan_destroy(P);
@@ -1364,6 +1373,7 @@ gw_status eps_core(gw_plan_s* P, int q, const c128* chi0, c128* E) {
     launch_zgemm<double>(N, N, N, mone, Vin, N, 0, OP_N, P->d_tmp, N, NN, OP_N, zero, E, N, NN, nw, st);
   } else {
     GW_TRY(sandwich(P, chi0, hw ? P->NK : q, -1.0, 1.0, E));
+    inject_timeout(P, "eps");
   }
   if (P->fp64) launch_axpby_identity<double>(N, E, NN, nw, 1.0, st);
   if (hw && P->p.head_wings == 1) {
@@ -1464,6 +1474,7 @@ gw_status sigma_core(gw_plan_s* P, int q, const c128* Wc, c128* sig, bool conjW 
         P->err = 1;
         return fail(ts, err);
       }
+      inject_timeout(P, "sigma");
     }
     launch_sigma_conv_chunk(kk0, nkk, nsig, NBd, P->p.nk, q, P->p.eps, P->d_mu, P->d_S_f, P->d_S_d, P->d_freq,
                             P->d_fw, nw, pref, sig, P->conv64, st, ktab);
@@ -1526,7 +1537,6 @@ gw_status g0w0_qlist(gw_plan_s* P, const std::vector<int>& qs_in, c128* sig_out,
     const int nq = (int)std::min<size_t>(P->qb, qs.size() - g0);
     const int* q = qs.data() + g0;
     const int* qp = partner.data() + g0;
-    GW_CUDA(cudaMemsetAsync(P->d_status, 0, sizeof(int), st));
     GW_TRY(chi0_prepare(P, q, nq));
     for (int j = 0; j < nq; ++j) GW_TRY(chi0_core(P, q[j], P->g_chi0 + j * slot));
     for (int j = 0; j < nq; ++j) GW_TRY(eps_core(P, q[j], P->g_chi0 + j * slot, P->g_E + j * slot));
@@ -1562,7 +1572,6 @@ gw_status gw_chi0(gw_plan P, int32_t sys, int32_t q, gw_complex* chi0_out) {
   cudaStream_t st = P->st;
   const size_t n = (size_t)P->N * P->N * P->nw;
   P->reset_timing();
-  GW_CUDA(cudaMemsetAsync(P->d_status, 0, sizeof(int), st));
   GW_TRY(chi0_core(P, q, P->d_chi0));
   GW_TRY(read_status(P, "gw_chi0"));
   GW_TRY(P->collect_timing());
@@ -1582,7 +1591,6 @@ gw_status gw_screen(gw_plan P, int32_t sys, int32_t q, gw_complex* wc_out) {
   cudaStream_t st = P->st;
   const long long NN = (long long)P->N * P->N;
   GW_TRY(eps_core(P, q, P->d_chi0, P->d_E));
-  GW_CUDA(cudaMemsetAsync(P->d_status, 0, sizeof(int), st));
   GW_TRY(invert(P, P->d_E, P->nw, P->d_work));
   if (q == 0 && P->p.head_wings == 2) GW_TRY(q0_average(P, P->d_E));
   GW_TRY(w_core(P, q, P->d_E, P->d_Wc));
@@ -1667,7 +1675,7 @@ gw_status gw_qp(gw_plan P, int32_t sys, const gw_complex* sigma, const double* d
   std::vector<int> conv(n);
   GW_CUDA(cudaMemcpyAsync(e_qp, d_e, n * sizeof(double), cudaMemcpyDeviceToHost, st));
   GW_CUDA(cudaMemcpyAsync(conv.data(), d_c, n * sizeof(int), cudaMemcpyDeviceToHost, st));
-  GW_CUDA(cudaStreamSynchronize(st));
+  GW_TRY(read_status(P, "gw_qp"));
   int nc = 0;
   for (int i = 0; i < n; ++i) nc += conv[i];
   if (n_conv) *n_conv = nc;
@@ -1774,7 +1782,7 @@ gw_status gw_qp_static(gw_plan P, int32_t sys, const gw_complex* sigma, const do
   int nc = 0;
   GW_CUDA(cudaMemcpyAsync(e_qp, sc->e_qp, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, st));
   GW_CUDA(cudaMemcpyAsync(&nc, &sc->n_conv, sizeof(int), cudaMemcpyDeviceToHost, st));
-  GW_CUDA(cudaStreamSynchronize(st));
+  GW_TRY(read_status(P, "gw_qp_static"));
   if (n_conv) *n_conv = nc;
   const int h = P->nocc - 1 - P->p.sigma_lo, l = P->nocc - P->p.sigma_lo;
   if (h >= 0 && h < P->nsig && l >= 0 && l < P->nsig) {
@@ -1948,6 +1956,7 @@ gw_status sigma_core_sur(gw_plan_s* P, int q, const c128* Wc_c, const c128* U, c
         P->err = 1;
         return fail(ts, err);
       }
+      inject_timeout(P, "sigma");
       c64* Pm = static_cast<c64*>(S.d_P);
       launch_zgemm<float>(R, k, N, c64{1, 0}, A, P->Kx, 0, OP_N, B32, k, 0, OP_N, c64{0, 0}, Pm, k, 0, 1, st);
       launch_sur_assemble<float>(R, nc, nw, k, S.d_jmap, S.d_Sc, Pm, coef, nf, Lmat, P->d_S_f, st);
@@ -1985,7 +1994,6 @@ gw_status g0w0_sur(gw_plan_s* P, c128* sig) {
   P->reset_timing();
   for (int q0 = 0; q0 < P->NK; q0 += S.qbs) {
     const int nq = std::min(S.qbs, P->NK - q0);
-    GW_CUDA(cudaMemsetAsync(P->d_status, 0, sizeof(int), st));
     {
       FreqView fv(P, nc, S.d_freq_c);
       std::vector<int> qg(nq);
@@ -2108,7 +2116,6 @@ gw_status gw_surrogate_modes(gw_plan P, int32_t sys, int32_t q, float* d_out, do
   cudaStream_t st = P->st;
   const int N = P->N, nw = P->nw;
   const long long NN = (long long)N * N;
-  GW_CUDA(cudaMemsetAsync(P->d_status, 0, sizeof(int), st));
   GW_TRY(eps_core(P, q, P->d_chi0, P->d_E));
   GW_CUDA(cudaMemcpyAsync(S.d_A1, P->d_E + S.coarse[0] * NN, sizeof(c128) * NN, cudaMemcpyDeviceToDevice, st));
   launch_axpby_identity<double>(N, S.d_A1, NN, 1, -1.0, st);
@@ -2148,7 +2155,6 @@ gw_status gw_surrogate_data(gw_plan P, int32_t sys, float* x_out, float* y_out, 
   P->reset_timing();
   for (int q0 = 0; q0 < P->NK; q0 += P->qb) {
     const int nq = std::min(P->qb, P->NK - q0);
-    GW_CUDA(cudaMemsetAsync(P->d_status, 0, sizeof(int), st));
     std::vector<int> qg(nq);
     for (int j = 0; j < nq; ++j) qg[j] = q0 + j;
     GW_TRY(chi0_prepare(P, qg.data(), nq));
