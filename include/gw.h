@@ -35,7 +35,7 @@
  *     GW_WORKSPACE_LIMIT    bytes of device memory one plan may allocate for its workspace
  *                           (default: no limit). An allocation that would pass it fails with
  *                           GW_ERR_NOMEM before cudaMalloc is called;
- *     GW_INJECT_TIMEOUT     for tests of a caller's error handling: the named products (eps, sigma)
+ *     GW_INJECT_TIMEOUT     for tests of a caller's error handling: the named products (sqrt, eps, sigma)
  *                           of a split precision report an expired wait although they ran.
  */
 #ifndef GW_H
@@ -147,7 +147,7 @@ size_t gw_problem_bytes(void);
  * system 0; gw_surrogate_enable is not available on a batch plan. n_sys in [1, 4096].
  * On success *out owns the workspace until gw_plan_destroy.
  * Errors: GW_ERR_ARG (bad sizes/pointers; for a batch the message names the system),
- * GW_ERR_NOMEM, GW_ERR_CUDA. */
+ * GW_ERR_NOMEM, GW_ERR_CUDA, GW_ERR_TIMEOUT. */
 gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw_plan* out);
 
 /* Release the plan and its workspace (waits for the plan's stream). NULL is a no-op. */

@@ -35,6 +35,13 @@ def expect_timeout(plan, call, *args, **kw):
     assert e.value.status == gw.GW_ERR_STATE
 
 
+def test_plan_creation_reports_its_products(plan_of):
+    from paper_2011_01400_gb300 import gw
+    with pytest.raises(gw.GwError) as e:
+        plan_of("sqrt")
+    assert e.value.status == gw.GW_ERR_TIMEOUT
+
+
 @pytest.mark.parametrize("prec", ["3xfp16", "3xtf32"])
 def test_screen_reports_its_first_products(plan_of, prec):
     from paper_2011_01400_gb300 import gw
