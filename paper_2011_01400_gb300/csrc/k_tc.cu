@@ -226,12 +226,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) k_tc(co
           const bool first = j == 0;
           if (first && gitem >= 2) {
             const uint32_t par = ((gitem >> 1) - 1) & 1;
-            if (!mbar_wait_cluster(&t1empty[b], par, p.status) || !mbar_wait_cluster(&t2empty[b], par, p.status)) {
+            if (!mbar_wait(PairBar{&t1empty[b]}, par, p.status) || !mbar_wait(PairBar{&t2empty[b]}, par, p.status)) {
               ok = false;
               break;
             }
           }
-          if (!mbar_wait_cluster(&full[s], ph, p.status)) { ok = false; break; }
+          if (!mbar_wait(PairBar{&full[s]}, ph, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t bbase = smem_u32(smem + s * STAGE);
           const uint64_t dB0 = sdesc(bbase), dB1 = sdesc(bbase + HALF);
