@@ -64,7 +64,7 @@ void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, cp
 template void launch_lri_halfT<double>(const LriGeom&, const double*, const c128*, c128*, c128*, cudaStream_t);
 
 // fp32 (split-precision plans): the same sums with the Fourier sum over the lattice vectors taken first,
-//   C(k)[(mu,i)][j] = sum_R e^{2 pi i k.R} C~(R)[(mu,i)][j]  (phases in FP64, sum in FP32),
+//   C(k)[(mu,i)][j] = sum_R e^{2 pi i k.R} C~(R)[(mu,i)][j]  (in FP64, rounded once),
 //   T1[k] = C(k) . c(k), batched over as many k as the staging holds.
 // One complex product per k instead of one per k and lattice vector onto T1: 64 k, 2 atoms of 200 ABFs and 39
 // functions, 78 bands, 7 lattice vectors 8.8 -> 2.6 ms.
@@ -73,27 +73,24 @@ namespace {
 // Ck[k - k0][e] for e < n (one atom's [(mu,i)][j]), k0 <= k < k0 + gridDim.y
 __global__ void k_lri_fourier(const __grid_constant__ LriGeom g, int k0, long long n, const double* __restrict__ ctil,
                               c64* __restrict__ Ck) {
-  __shared__ float cs[64], sn[64];
+  __shared__ double cs[64], sn[64];
   const int k = k0 + blockIdx.y;
   if (threadIdx.x < g.nR) {
     const int r = threadIdx.x, k3 = k % g.nk[2], k2 = (k / g.nk[2]) % g.nk[1], k1 = k / (g.nk[1] * g.nk[2]);
     const double ph = 2.0 * (((double)k1 / g.nk[0] + g.koff[0]) * g.R[r][0] +
                              ((double)k2 / g.nk[1] + g.koff[1]) * g.R[r][1] +
                              ((double)k3 / g.nk[2] + g.koff[2]) * g.R[r][2]);
-    double s, c;
-    sincospi(ph, &s, &c);
-    cs[r] = (float)c;
-    sn[r] = (float)s;
+    sincospi(ph, &sn[r], &cs[r]);
   }
   __syncthreads();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    float re = 0.f, im = 0.f;
+    double re = 0.0, im = 0.0;
     for (int r = 0; r < g.nR; ++r) {
-      const float x = (float)ctil[r * n + e];
-      re = fmaf(x, cs[r], re);
-      im = fmaf(x, sn[r], im);
+      const double x = ctil[r * n + e];
+      re = fma(x, cs[r], re);
+      im = fma(x, sn[r], im);
     }
-    Ck[blockIdx.y * n + e] = c64{re, im};
+    Ck[blockIdx.y * n + e] = c64{(float)re, (float)im};
   }
 }
 
