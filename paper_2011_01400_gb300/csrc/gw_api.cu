@@ -864,7 +864,7 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
         P->d_Apl[i] = pp;
       }
       const size_t we = (size_t)nw * N * 2 * P->Kx * (P->prec == GW_3XTF32 ? 4 : 2);
-      for (int i = 0; i < (P->prec == GW_3XTF32 ? 4 : 6); ++i) {
+      for (int i = 0; i < 4; ++i) {
         uint8_t* pp;
         ALLOC(pp, we);
         P->d_Wpl.b[i] = pp;
@@ -1461,7 +1461,7 @@ gw_status sigma_core(gw_plan_s* P, int q, const c128* Wc, c128* sig, bool conjW 
       a.Kpad = P->Kx;
       a.nw = nw;
       a.raw = reinterpret_cast<const float*>(A);
-      for (int i = 0; i < 6; ++i) a.bpl[i] = P->d_Wpl.b[i];
+      for (int i = 0; i < 4; ++i) a.bpl[i] = P->d_Wpl.b[i];
       a.S = P->d_S_f;
       a.apl[0] = P->d_Apl[0];
       a.apl[1] = P->d_Apl[1];
@@ -1943,7 +1943,7 @@ gw_status sigma_core_sur(gw_plan_s* P, int q, const c128* Wc_c, const c128* U, c
       a.Kpad = P->Kx;
       a.nw = nc;
       a.raw = reinterpret_cast<const float*>(A);
-      for (int i = 0; i < 6; ++i) a.bpl[i] = P->d_Wpl.b[i];
+      for (int i = 0; i < 4; ++i) a.bpl[i] = P->d_Wpl.b[i];
       a.S = S.d_Sc;
       a.apl[0] = P->d_Apl[0];
       a.apl[1] = P->d_Apl[1];

@@ -147,7 +147,7 @@ void launch_qp(int NK, int nsig, int NBd, int sig_lo, int nw, const c128* sigma,
 
 // k_tc.cu -- tcgen05 split-precision Sigma_c contraction (and the chi0 / W^c plane helpers)
 struct PlaneSet {
-  void* b[6];       // B1 pieces then B2 pieces
+  void* b[4];       // two B1 pieces then two B2 pieces
 };
 struct TcSigmaArgs {
   int R;            // rows a_r = C^mu_{nm}(k, k-q) of this chunk
@@ -155,7 +155,7 @@ struct TcSigmaArgs {
   int Kpad;         // n_aux rounded up to 32 (K = mu)
   int nw;
   const float* raw; // [R][2*Kpad] fp32 (re, im) of a_r (zero beyond n_aux)
-  const void* bpl[6];  // W^c planes [nw*N][2*Kpad] (B1 pieces then B2 pieces)
+  const void* bpl[4];  // W^c planes [nw*N][2*Kpad] (two B1 pieces then two B2 pieces)
   void* apl[2];     // workspace: A pieces [R][2*Kpad] (bf16 or tf32), written by tc_sigma_run from raw
   float* S;         // [R][nw] accumulated (zeroed by the caller)
   int tf32;

@@ -354,8 +354,7 @@ __global__ void k_a_planes(long long n, const float* __restrict__ raw, void* p0,
 
 // B planes of W^c (conj: of conj(W^c)) for the Sigma contraction: row (j, nu), K index 2 mu + {0, 1}:
 // B1 = split(Re W_{nu mu}, Im W_{nu mu}), B2 = split(-Im, Re); mu >= N is zero padding.
-__global__ void k_w_planes(int N, int nw, int Kpad, const c128* __restrict__ Wc, PlaneSet P, int tf32, int np,
-                           int conj) {
+__global__ void k_w_planes(int N, int nw, int Kpad, const c128* __restrict__ Wc, PlaneSet P, int tf32, int conj) {
   const long long total = (long long)nw * N * Kpad;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
@@ -383,13 +382,8 @@ __global__ void k_w_planes(int N, int nw, int Kpad, const c128* __restrict__ Wc,
         const float2 hf = __bfloat1622float2(h);
         const float r0 = v[0] - hf.x, r1 = v[1] - hf.y;
         const __nv_bfloat162 mm = __floats2bfloat162_rn(r0, r1);
-        *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(P.b[np * half]) + o) = h;
-        *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(P.b[np * half + 1]) + o) = mm;
-        if (np == 3) {
-          const float2 mf = __bfloat1622float2(mm);
-          const __nv_bfloat162 l = __floats2bfloat162_rn(r0 - mf.x, r1 - mf.y);
-          *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(P.b[np * half + 2]) + o) = l;
-        }
+        *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(P.b[2 * half]) + o) = h;
+        *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(P.b[2 * half + 1]) + o) = mm;
       }
     }
   }
@@ -530,7 +524,7 @@ gw_status tc_sigma_run(const TcSigmaArgs& a, cudaStream_t st, std::string& err) 
 
 void tc_w_planes(int N, int nw, int Kpad, const c128* Wc, const PlaneSet& P, int tf32, cudaStream_t st, int conj) {
   const long long total = (long long)nw * N * Kpad;
-  ++::gw::g_launch_count, k_w_planes<<<std::min<long long>((total + 255) / 256, 152 * 64), 256, 0, st>>>(N, nw, Kpad, Wc, P, tf32, 2, conj);
+  ++::gw::g_launch_count, k_w_planes<<<std::min<long long>((total + 255) / 256, 152 * 64), 256, 0, st>>>(N, nw, Kpad, Wc, P, tf32, conj);
 }
 
 void tc_herm_fill(int N, int nw, c128* chi0, cudaStream_t st) {
