@@ -352,6 +352,7 @@ template <typename T> gw_status dalloc(gw_plan_s* P, T** ptr, size_t count) {
   const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
   if (P->measuring) {
     P->arena_need += arena_round(bytes);
+    *ptr = nullptr;
     return GW_OK;
   }
   if (P->ws_limit && P->ws_bytes + bytes > P->ws_limit)
