@@ -970,12 +970,13 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
   }
   CK(cudaMemcpyAsync(&P->mu, P->d_mu, sizeof(double), cudaMemcpyDeviceToHost, st));
   // half-transformed LRI coefficients
+  const c128* evec = reinterpret_cast<const c128*>(prob->evec);
   if (P->fp64)
-    launch_lri_halfT<double>(g, prob->ctil_R, reinterpret_cast<const c128*>(prob->evec),
-                             static_cast<c128*>(P->d_T1), nullptr, st);
-  else
-    launch_lri_halfT<float>(g, prob->ctil_R, reinterpret_cast<const c128*>(prob->evec), static_cast<c64*>(P->d_T1),
-                            nullptr, st);
+    launch_lri_halfT<double>(g, prob->ctil_R, evec, evec, static_cast<c128*>(P->d_T1), st);
+  else {
+    launch_convert((long long)P->NK * P->NB * P->NBd, evec, P->d_evec32, st);
+    launch_lri_halfT<float>(g, prob->ctil_R, evec, P->d_evec32, static_cast<c64*>(P->d_T1), st);
+  }
   if ((s = check_launch(P, "lri_halfT")) != GW_OK) return cleanup(s);
   // time-reversal symmetry of the inputs, when the caller declares it
   if (prob->time_reversal) {
@@ -1043,7 +1044,6 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
     launch_rank1(N, P->d_Vh, P->d_x1, std::sqrt(std::max(P->h_v1, 0.0)), st);
   }
   if (!P->fp64) {
-    launch_convert((long long)P->NK * P->NB * P->NBd, reinterpret_cast<const c128*>(prob->evec), P->d_evec32, st);
     // pieces of V^1/2 (d_hmax holds the largest elements meanwhile)
     auto pieces = [&](const c128* V, int mats, size_t m0) {
       const size_t o = m0 * N * 2 * P->Kx;

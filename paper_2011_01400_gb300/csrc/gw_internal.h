@@ -50,7 +50,7 @@ enum Op { OP_N = 0, OP_T = 1, OP_C = 2, OP_CONJ = 3 };   // as is, transpose, co
 
 // k_lri.cu -- step (a)
 // T1_A[k][mu][i][b] = sum_R e^{2 pi i k.R} sum_j C~_A[R][mu][i][j] c[k][j][b]              (mu, i on A)
-// T2_A[k][mu][j][a] = sum_R e^{-2 pi i k.R} sum_i C~_A[R][mu][j][i] conj(c[k][i][a])      (mu, j on A)
+// evec: the eigenvectors, evec_t: the same in T
 struct LriGeom {
   int n_atoms, NK, NB, NBd, N, nR;
   int nk[3];
@@ -62,7 +62,7 @@ struct LriGeom {
   int R[64][3];
 };
 template <typename T>
-void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, cplx<T>* T1, cplx<T>* T2,
+void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, const cplx<T>* evec_t, cplx<T>* T1,
                       cudaStream_t st);
 
 // M^mu_{ab}(k', q) for a in [a0, a0+na) at k'+q and b in [b0, b0+nb) at k', for the k' of each row block.

@@ -53,7 +53,7 @@ __global__ void k_lri_halfT(const __grid_constant__ LriGeom g, const double* __r
 }
 
 template <typename T>
-void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, cplx<T>* T1, cplx<T>* /*T2*/,
+void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, const cplx<T>* /*evec_t*/, cplx<T>* T1,
                       cudaStream_t st) {
   for (int A = 0; A < g.n_atoms; ++A) {
     long long total = (long long)g.NK * g.atom_nx[A] * g.atom_nb[A] * g.NBd;
@@ -61,7 +61,7 @@ void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, cp
     ++::gw::g_launch_count, k_lri_halfT<T><<<blocks, 256, 0, st>>>(g, ctil, evec, T1, A);
   }
 }
-template void launch_lri_halfT<double>(const LriGeom&, const double*, const c128*, c128*, c128*, cudaStream_t);
+template void launch_lri_halfT<double>(const LriGeom&, const double*, const c128*, const c128*, c128*, cudaStream_t);
 
 // fp32 (split-precision plans): the same sums with the Fourier sum over the lattice vectors taken first,
 //   C(k)[(mu,i)][j] = sum_R e^{2 pi i k.R} C~(R)[(mu,i)][j]  (in FP64, rounded once),
@@ -97,20 +97,17 @@ __global__ void k_lri_fourier(const __grid_constant__ LriGeom g, int k0, long lo
 }  // namespace
 
 template <>
-void launch_lri_halfT<float>(const LriGeom& g, const double* ctil, const c128* evec, c64* T1, c64* /*T2*/,
+void launch_lri_halfT<float>(const LriGeom& g, const double* ctil, const c128* evec, const c64* evec_t, c64* T1,
                              cudaStream_t st) {
   const long long per_k = (long long)g.NB * g.NBd;
   long long amax = 0;
   for (int A = 0; A < g.n_atoms; ++A) amax = std::max(amax, (long long)g.atom_nx[A] * g.atom_nb[A] * g.NB);
   const int kc = (int)std::max<long long>(1, std::min<long long>(g.NK, (256LL << 20) / (amax * (long long)sizeof(c64))));
-  c64 *c32 = nullptr, *Ck = nullptr;
-  ::gw::g_alloc_count += 2;
-  if (cudaMallocAsync(&c32, sizeof(c64) * per_k * g.NK, st) != cudaSuccess ||
-      cudaMallocAsync(&Ck, sizeof(c64) * amax * kc, st) != cudaSuccess) {
+  c64* Ck = nullptr;
+  ++::gw::g_alloc_count;
+  if (cudaMallocAsync(&Ck, sizeof(c64) * amax * kc, st) != cudaSuccess) {
     // fall back to the direct kernel (same sums, FP64 arithmetic) when the staging does not fit
     cudaGetLastError();
-    if (c32) cudaFreeAsync(c32, st);
-    if (Ck) cudaFreeAsync(Ck, st);
     for (int A = 0; A < g.n_atoms; ++A) {
       long long total = (long long)g.NK * g.atom_nx[A] * g.atom_nb[A] * g.NBd;
       int blocks = (int)std::min<long long>((total + 255) / 256, 152LL * 64);
@@ -118,18 +115,16 @@ void launch_lri_halfT<float>(const LriGeom& g, const double* ctil, const c128* e
     }
     return;
   }
-  launch_convert(per_k * g.NK, evec, c32, st);
   for (int A = 0; A < g.n_atoms; ++A) {
     const long long rows = (long long)g.atom_nx[A] * g.atom_nb[A], n = rows * g.NB;
     for (int k0 = 0; k0 < g.NK; k0 += kc) {
       const int nk = std::min(kc, g.NK - k0);
       ++::gw::g_launch_count, k_lri_fourier<<<dim3((unsigned)std::min<long long>((n + 255) / 256, 1024), nk), 256, 0, st>>>(
           g, k0, n, ctil + g.ctil_off[A], Ck);
-      launch_zgemm<float>((int)rows, g.NBd, g.NB, c64{1, 0}, Ck, g.NB, n, OP_N, c32 + k0 * per_k, g.NBd, per_k, OP_N,
+      launch_zgemm<float>((int)rows, g.NBd, g.NB, c64{1, 0}, Ck, g.NB, n, OP_N, evec_t + k0 * per_k, g.NBd, per_k, OP_N,
                           c64{0, 0}, T1 + g.t_off[A] + k0 * rows * g.NBd, g.NBd, rows * g.NBd, nk, st);
     }
   }
-  cudaFreeAsync(c32, st);
   cudaFreeAsync(Ck, st);
 }
 

@@ -24,3 +24,17 @@ def test_planes(prec, size):
     gw.gw_plan_destroy(plan)
     mats, plane = 6 * 16 * nw * n * n, size * nw * n * 2 * n
     assert held <= mats + 4 * plane + 64 * 2 ** 20        # (pieces and tables of one q: 30 MB; a plane: 67 or 134 MB)
+
+
+def test_allocations_of_a_new_plan():
+    """One for the plan's buffers, one for the half transform's staging, three for the work lists of the products; the
+    eigenvectors are converted once, into the plan."""
+    pytest.importorskip("torch")
+    from paper_2011_01400_gb300 import gw
+    s = make_system("cfg0", seed=1, head_wings=0, trs=False)
+    pb = gw.Problem(s, "3xfp16")
+    n = gw.gw_device_allocations()
+    plan = gw.gw_plan_create(pb.prob)
+    n = gw.gw_device_allocations() - n
+    gw.gw_plan_destroy(plan)
+    assert n == 5
