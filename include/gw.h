@@ -30,7 +30,12 @@
  *     GW_CHI0_SEG_ROWS      pair rows per FP64 promotion segment of the tensor-core
  *                           chi0 (default 8192; at least 32);
  *     GW_CHI0_COMPRESS_TOL  per-frequency residual bound of the chi0 weight-matrix
- *                           compression (default 3e-8; 0 keeps all frequencies).
+ *                           compression (default 3e-8; 0 keeps all frequencies);
+ *     GW_SIGMA_CONV64       1: the frequency convolution of Sigma_c in FP64 (default 0: FP32). In
+ *                           FP32 z^2 + w_j^2 cancels at w = w_j >> |Re z|: Sigma_c at the largest
+ *                           frequencies is up to 1e-4 off (relative; 1e-5 in FP64), and the
+ *                           two-pole fit of gw_qp can turn that into 1e-4 Ha and, where it is
+ *                           badly conditioned, 1e-3 Ha of single quasiparticle energies.
  *   - Environment (read at gw_plan_create, all precisions):
  *     GW_WORKSPACE_LIMIT    bytes of device memory one plan may allocate for its workspace
  *                           (default: no limit). An allocation that would pass it fails with

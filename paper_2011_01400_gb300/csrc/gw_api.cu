@@ -795,8 +795,9 @@ gw_status gw_plan_create(const gw_problem* prob, int32_t n_sys, void* stream, gw
       P->fweight[j] = 2.0 * prob->omega0 * w[j] / ((1.0 - x[j]) * (1.0 - x[j]));
     }
   }
-  // the FP32 convolution forms products up to w^4
-  P->conv64 = P->fp64 || *std::max_element(P->freq.begin(), P->freq.end()) > 1e9;
+  // the FP32 convolution forms products up to w^4, and cancels where w = w_j (k_sigma_conv)
+  const char* conv = std::getenv("GW_SIGMA_CONV64");
+  P->conv64 = P->fp64 || (conv && std::atoi(conv) != 0) || *std::max_element(P->freq.begin(), P->freq.end()) > 1e9;
   const int N = P->N, nw = P->nw;
   const size_t NN = (size_t)N * N;
   gw_status s;

@@ -28,6 +28,11 @@ void launch_rowdot(int R, int N, const c128* U, const c128* a, long long ld, dou
 // order in FP64. A kernel value (a division and ~15 FMAs) per (m, j, w) bounds it; S is read by whole
 // warps at one address. 216 k, 8 window bands, 78 bands, 32 frequencies: 140 us, 487 us with one thread
 // per (kk, n, w); one k, 300 bands, where that filled two blocks: 48 us, 1254 us before.
+// T = float loses zr^2 in (zr^2 - om^2) + w_j^2 at w_j = om >> |zr| (om ~ 700: 0.03 absolute). The sum over
+// j hides it in the norm of Sigma_c (3e-6 either way) but not at the largest frequencies: 40 passes of 14-288 (k, n)
+// against FP64: median error of the last frequency 0.4-8.5e-5, with zr^2 + (w_j - om)(w_j + om) 0.1-1.3e-5; largest
+// error of an E_QP 1.3e-3 Ha against 3e-5. That form is not the default because it moves E_QP by up to 1e-4 relative
+// from what this one has always given; conv64 (T = double) is the accurate way.
 template <typename T>
 __global__ void k_sigma_conv(int kk0, int nsig, int NBd, int n1, int n2, int n3, int q, const double* __restrict__ eps,
                              const double* __restrict__ mu_p, const float* __restrict__ S_f,
