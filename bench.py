@@ -752,9 +752,9 @@ def run_device(args, system, world, rank):
         # measured FP64 GEMM (4 N^3 flops per (q, w) matrix: N^3 / 2 complex multiply-adds)
         peak64 = fp64_gemm_peak(torch)
         nq = q_computed(s)
-        chol_flops = 4.0 * s.n_aux ** 3 * s.n_freq * nq
+        inv_flops = 4.0 * s.n_aux ** 3 * s.n_freq * nq
         line["fp64_peak"] = dict(dgemm_tflops=peak64, method="cuBLAS DGEMM via torch.matmul, 4096^3, best of 5, "
-                                                           "CUDA events", cholesky_flops_per_step=chol_flops)
+                                                           "CUDA events", inverse_flops_per_step=inv_flops)
     # the learned surrogate and the batch of uneven systems: part of the default N = 1 line
     if args.surrogate or (world == 1 and not args.no_extras):
         line["surrogate"] = surrogate_bench(args, gw, torch)
