@@ -64,33 +64,57 @@ void launch_lri_halfT(const LriGeom& g, const double* ctil, const c128* evec, co
 template void launch_lri_halfT<double>(const LriGeom&, const double*, const c128*, const c128*, c128*, cudaStream_t);
 
 // fp32 (split-precision plans): the same sums with the Fourier sum over the lattice vectors taken first,
-//   C(k)[(mu,i)][j] = sum_R e^{2 pi i k.R} C~(R)[(mu,i)][j]  (in FP64, rounded once),
+//   C(k)[(mu,i)][j] = sum_R e^{2 pi i k.R} C~(R)[(mu,i)][j]  (to 2^-46, rounded once),
 //   T1[k] = C(k) . c(k), batched over as many k as the staging holds.
 // One complex product per k instead of one per k and lattice vector onto T1: 64 k, 2 atoms of 200 ABFs and 39
-// functions, 78 bands, 7 lattice vectors 8.8 -> 2.6 ms.
+// functions, 78 bands, 7 lattice vectors 8.8 -> 2.0 ms.
 namespace {
 
-// Ck[k - k0][e] for e < n (one atom's [(mu,i)][j]), k0 <= k < k0 + gridDim.y
-__global__ void k_lri_fourier(const __grid_constant__ LriGeom g, int k0, long long n, const double* __restrict__ ctil,
-                              c64* __restrict__ Ck) {
-  __shared__ double cs[64], sn[64];
-  const int k = k0 + blockIdx.y;
-  if (threadIdx.x < g.nR) {
-    const int r = threadIdx.x, k3 = k % g.nk[2], k2 = (k / g.nk[2]) % g.nk[1], k1 = k / (g.nk[1] * g.nk[2]);
-    const double ph = 2.0 * (((double)k1 / g.nk[0] + g.koff[0]) * g.R[r][0] +
-                             ((double)k2 / g.nk[1] + g.koff[1]) * g.R[r][1] +
-                             ((double)k3 / g.nk[2] + g.koff[2]) * g.R[r][2]);
-    sincospi(ph, &sn[r], &cs[r]);
+// Ck[k - k0][e] for e < n (one atom's [(mu,i)][j]), LF_K consecutive k per block. The sums run in pairs of floats
+// (products and additions with their rounding errors, 2^-46 of the terms): on the FP64 units, 2 multiply-adds
+// per clock and SM, they took 2.7 ms of a plan of 64 k, 2 atoms, 200 ABFs, 39 functions, 78 bands, 7 vectors; 0.93 ms now.
+constexpr int LF_K = 8;
+struct Pair32 {
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float xh, float xl, float ch, float cl) {   // += (xh + xl) (ch + cl)
+    const float p = __fmul_rn(xh, ch);
+    const float e = fmaf(xh, cl, fmaf(xl, ch, fmaf(xh, ch, -p)));
+    const float s = __fadd_rn(h, p), b = __fsub_rn(s, h);
+    l += __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(p, b)) + e;
+    h = s;
+  }
+};
+__global__ void __launch_bounds__(256) k_lri_fourier(const __grid_constant__ LriGeom g, int k0, int nk, long long n,
+                                                     const double* __restrict__ ctil, c64* __restrict__ Ck) {
+  __shared__ float4 ph[64][LF_K];      // cos and sin, each as a pair
+  const int kb = blockIdx.y * LF_K;
+  for (int i = threadIdx.x; i < g.nR * LF_K; i += blockDim.x) {
+    const int r = i / LF_K, k = k0 + min(kb + i % LF_K, nk - 1);
+    const int k3 = k % g.nk[2], k2 = (k / g.nk[2]) % g.nk[1], k1 = k / (g.nk[1] * g.nk[2]);
+    const double x = 2.0 * (((double)k1 / g.nk[0] + g.koff[0]) * g.R[r][0] +
+                            ((double)k2 / g.nk[1] + g.koff[1]) * g.R[r][1] +
+                            ((double)k3 / g.nk[2] + g.koff[2]) * g.R[r][2]);
+    double s, c;
+    sincospi(x, &s, &c);
+    const float ch = (float)c, sh = (float)s;
+    ph[r][i % LF_K] = make_float4(ch, (float)(c - ch), sh, (float)(s - sh));
   }
   __syncthreads();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    double re = 0.0, im = 0.0;
+    Pair32 re[LF_K], im[LF_K];
     for (int r = 0; r < g.nR; ++r) {
       const double x = ctil[r * n + e];
-      re = fma(x, cs[r], re);
-      im = fma(x, sn[r], im);
+      const float xh = (float)x, xl = (float)(x - xh);
+#pragma unroll
+      for (int k = 0; k < LF_K; ++k) {
+        const float4 f = ph[r][k];
+        re[k].add(xh, xl, f.x, f.y);
+        im[k].add(xh, xl, f.z, f.w);
+      }
     }
-    Ck[blockIdx.y * n + e] = c64{(float)re, (float)im};
+#pragma unroll
+    for (int k = 0; k < LF_K; ++k)
+      if (kb + k < nk) Ck[(kb + k) * n + e] = c64{re[k].h + re[k].l, im[k].h + im[k].l};
   }
 }
 
@@ -119,8 +143,8 @@ void launch_lri_halfT<float>(const LriGeom& g, const double* ctil, const c128* e
     const long long rows = (long long)g.atom_nx[A] * g.atom_nb[A], n = rows * g.NB;
     for (int k0 = 0; k0 < g.NK; k0 += kc) {
       const int nk = std::min(kc, g.NK - k0);
-      ++::gw::g_launch_count, k_lri_fourier<<<dim3((unsigned)std::min<long long>((n + 255) / 256, 1024), nk), 256, 0, st>>>(
-          g, k0, n, ctil + g.ctil_off[A], Ck);
+      const dim3 grid((unsigned)std::min<long long>((n + 255) / 256, 1024), (nk + LF_K - 1) / LF_K);
+      ++::gw::g_launch_count, k_lri_fourier<<<grid, 256, 0, st>>>(g, k0, nk, n, ctil + g.ctil_off[A], Ck);
       launch_zgemm<float>((int)rows, g.NBd, g.NB, c64{1, 0}, Ck, g.NB, n, OP_N, evec_t + k0 * per_k, g.NBd, per_k, OP_N,
                           c64{0, 0}, T1 + g.t_off[A] + k0 * rows * g.NBd, g.NBd, rows * g.NBd, nk, st);
     }
