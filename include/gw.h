@@ -64,6 +64,8 @@ typedef enum {
   GW_ERR_UNSUPPORTED = 7 /* valid request that the library does not implement          */
 } gw_status;
 
+/* The split precisions name the pieces of chi0 and Sigma_c; the screen products take two FP16 pieces with one
+ * power-of-two scale per matrix in all of them (22 bits, as two TF32 pieces). */
 typedef enum {
   GW_FP64 = 0,    /* plain method: every contraction in FP64 on CUDA cores          */
   GW_3XTF32 = 1,  /* contractions as 3 TF32 split products on tcgen05, FP32 accum.   */
