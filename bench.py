@@ -30,7 +30,7 @@ METRIC = "G0W0 Σc time-to-solution & χ0 TFLOP/s: split-prec vs FP64 on 1 GB300
 # ncu capture of k_chi0 (3xFP16) on the cfg1 shape with a 4x4x4 k mesh (the third chi0 launch of a
 # pass; its summary is kept with the other profiles). The reads stream the operand planes of every
 # k and grow with the k count; the writes are the FP64 output rows, independent of it.
-CHI0_DRAM_CAPTURE = dict(prec="3xfp16", n_k=64, n_aux=400, read=271.424512e6, write=39.426304e6)
+CHI0_DRAM_CAPTURE = dict(prec="3xfp16", n_k=64, n_aux=400, read=268.078336e6, write=34.337024e6)
 WORKLOADS = {
     "cfg0": "tiny synthetic insulator: 2x2x2 k, 2 atoms, 32 NAO, 32 bands (4 occ), 96 ABF, 16 imaginary frequencies",
     "cfg1": "Si-like 2-atom fcc cell: 6x6x6 k (216 k, 216 q), 78 NAO, 78 bands (4 occ), 400 ABF, 32 imaginary "

@@ -23,15 +23,16 @@
 // Scaling: an element 2^m below its row's largest is known to m bits less, so the error of a matrix D A D,
 // D diagonal, would grow with the spread of D (which it does not in FP64 elimination): 5e-13 at a spread
 // of 1e4, 4e-11 at 1e6. Rows and columns are therefore scaled by powers of two of the diagonal first, which is
-// exact and leaves 4e-16 at every spread (N = 200, against 5e-16 for FP64 Cholesky). eps~ with its
-// diagonal in [1, 4), the usual one, is not touched: the pass costs the two launches.
+// exact and leaves 4e-16 at every spread (N = 200, against 5e-16 for FP64 Cholesky). Elements between rows
+// whose diagonal is in [1, 4) are not touched. It costs 1% of a screening call (16 matrices of N = 1200 with a
+// larger diagonal: 0.13 of 15.3 ms).
 //
 // Why: the chip does ~2 FP64 FMA per clock and SM (1.1 TFLOP/s by cuBLAS DGEMM) and the 4 N^3 flops
 // of an inverse bound the screening by that; 28 FP16 products of the tensor cores are ~25 times
 // faster than one FP64 one. What is left in FP64 is one addition per element and pivot block, and
 // the factor of the 32 x 32 pivot blocks. Every size is spread over the whole chip (a CTA per 64 rows
 // of a matrix). Measured against one block per matrix with FP64 FMAs throughout: 1152 matrices of
-// N = 400 332 -> 47 ms, 32 of them 44 -> 2.1 ms, 16 of N = 1200 1004 -> 10.6 ms, 32 of N = 96 1.5 -> 0.4 ms;
+// N = 400 332 -> 47 ms, 32 of them 44 -> 2.1 ms, 16 of N = 1200 1004 -> 10.7 ms, 32 of N = 96 1.5 -> 0.4 ms;
 // the error against a refined inverse is the same (N = 400: 3.7e-16 and 5.6e-16 before at kappa = 3,
 // 4.7e-10 and 6.5e-10 before at kappa = 2e7). Two thirds of it are the updates, which take ~9 us per 64 x 64
 // tile: the products need 2, the FP64 conversions and additions of the epilogue 3, the rest is latency
@@ -166,30 +167,19 @@ __global__ void k_inv_exps(int N, const c128* __restrict__ Aall, long long strid
   sc[(long long)blockIdx.y * N + i] = d > 0.0 && isfinite(d) ? -(ilogb(d) >> 1) : 0;
 }
 
-// the scales of the 32 memory rows from j0 and of the 32 columns from i0; false if all are zero
-__device__ __forceinline__ bool tile_scales(int N, const int* __restrict__ sc, int j0, int i0, int (&se)[64]) {
-  const int t = threadIdx.y * 32 + threadIdx.x, r = t < 32 ? j0 + t : i0 + t - 32;
-  int s = 0;
-  if (t < 64) {
-    s = r < N ? sc[r] : 0;
-    se[t] = s;
-  }
-  return __syncthreads_or(s) != 0;
-}
-
-// The kept triangle of A; tiles whose scales are all zero are not touched
-__global__ void k_inv_scale(int N, c128* __restrict__ Aall, long long stride, const int* __restrict__ sc) {
-  __shared__ int se[64];
+// The kept triangle of A; elements with nothing to scale are not touched
+__global__ void k_inv_scale(int N, c128* __restrict__ Aall, long long stride, const int* __restrict__ scall) {
   if (blockIdx.x < blockIdx.y) return;
   c128* A = Aall + blockIdx.z * stride;
-  const int j0 = blockIdx.y * 32, i0 = blockIdx.x * 32;
-  if (!tile_scales(N, sc + (long long)blockIdx.z * N, j0, i0, se)) return;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int j = j0 + r, i = i0 + threadIdx.x;
-    if (j < N && i < N && i >= j) {
-      const double fj = pow2(se[r]), fi = pow2(se[32 + threadIdx.x]);   // (one after the other: no overflow)
+  const int* sc = scall + (long long)blockIdx.z * N;
+  const int j0 = blockIdx.y * 32, i = blockIdx.x * 32 + threadIdx.x;
+  if (i >= N) return;
+  const int si = sc[i];
+  for (int j = j0 + threadIdx.y; j < min(N, j0 + 32); j += blockDim.y) {
+    const int sj = sc[j];
+    if (i >= j && (si | sj) != 0) {
       c128& a = A[(long long)j * N + i];
-      a = c128{a.re * fj * fi, a.im * fj * fi};
+      a = c128{a.re * pow2(sj) * pow2(si), a.im * pow2(sj) * pow2(si)};   // (one after the other: no overflow)
     }
   }
 }
@@ -664,18 +654,17 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_inv_update(const __grid_cons
 }
 
 // A := -B - I in full from the kept triangle, the scales of A undone
-__global__ void k_inv_finish(int N, c128* __restrict__ Aall, long long stride, const int* __restrict__ sc) {
+__global__ void k_inv_finish(int N, c128* __restrict__ Aall, long long stride, const int* __restrict__ scall) {
   __shared__ c128 tt[32][33];
-  __shared__ int se[64];
   if (blockIdx.x < blockIdx.y) return;
   c128* A = Aall + blockIdx.z * stride;
+  const int* sc = scall + (long long)blockIdx.z * N;
   const int j0 = blockIdx.y * 32, i0 = blockIdx.x * 32;     // memory rows j, columns i >= j
-  tile_scales(N, sc + (long long)blockIdx.z * N, j0, i0, se);
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int j = j0 + r, i = i0 + threadIdx.x;
     if (j < N && i < N && i >= j) {
       c128 v = A[(long long)j * N + i];
-      const double fj = pow2(se[r]), fi = pow2(se[32 + threadIdx.x]);
+      const double fj = pow2(sc[j]), fi = pow2(sc[i]);
       v = c128{v.re * fj * fi, v.im * fj * fi};
       const c128 o = i == j ? c128{-v.re - 1.0, 0.0} : c128{-v.re, -v.im};
       A[(long long)j * N + i] = o;
