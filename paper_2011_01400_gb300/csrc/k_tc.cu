@@ -22,8 +22,9 @@
 // Pairs of CTAs (clusters of two, cta_group::2): an item is 256 rows, 128 in each CTA, against the same 64
 // columns; CTA 0 holds B1, CTA 1 B2, and one MMA (M = 256, N = 128) reads both. Shared memory bounds the
 // kernel: a stage of 12 MMAs reads 8 KB of operands per MMA and CTA when a CTA works alone (96 KB, and 64 KB
-// written by TMA: 1280 of its 1540 clocks), 6 KB in a pair (72 KB and 48 KB: 940 of 1360). Measured, per q:
-// 216 k, N = 400, 32 frequencies 8.15 -> 7.53 ms; one k, N = 1600, TF32 4.90 -> 3.34 ms.
+// written by TMA: 1280 of its 1540 clocks), 6 KB in a pair (72 KB and 48 KB: 940 of 1275). Measured, per q:
+// 216 k, N = 400, 32 frequencies 8.15 -> 7.53 ms; one k, N = 1600, TF32 4.90 -> 3.34 ms; and the issue loop per
+// segment, without tests for its ends in every stage, 0.37 and 0.17 ms off the two whole calls (9.37 and 4.30 ms).
 //
 // Work distribution: one pair of CTAs per two SMs, each walking the work items (row block, frequency,
 // column block; column block fastest, so that concurrent pairs share their W^c tiles in L2); all pipelines
