@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("one_sign", [False, True])
 @pytest.mark.parametrize("prec,pieces,adds", [("3xtf32", 2.0 ** -20, 128), ("3xfp16", 2.0 ** -16, 64)])
-@pytest.mark.parametrize("n_aux", [1000, 1600])
+# 512 ABFs are one segment (16 or 32 stages), 514 and 544 one stage more
+@pytest.mark.parametrize("n_aux", [510, 512, 514, 544, 1000, 1600])
 def test_error_of_the_accumulator(one_sign, prec, pieces, adds, n_aux):
     torch = pytest.importorskip("torch")
     from paper_2011_01400_gb300 import gw
