@@ -1,5 +1,5 @@
 // FP64 inversion of the batched Hermitian positive definite eps~ (step c), A := A^{-1} - I, with its
-// rank-32 updates on the FP16 tensor cores as exact integer products.
+// rank-32 updates on the FP16 tensor cores as products of integer digits.
 //
 // Method: block elimination over pivot blocks P of 32 indices, in place. With the Cholesky factor
 // L of B_PP and W = L^{-1},
@@ -64,7 +64,7 @@ constexpr int W_PLANE = 2 * PB * ROWB;   // one digit of W, Re / Im rows stacked
 constexpr int R_PLANE = PB * ROWB;       // one digit of W^H as right rows
 constexpr int E_BAD = 1 << 20;           // exponent of a row with an infinity or a NaN
 
-// ---- exact splitting -------------------------------------------------------------------------
+// ---- splitting into digits----------------------------------------------------------------------
 
 // exponent field of the largest of 8 doubles
 __device__ __forceinline__ int max_field(const double (&v)[8]) {
